@@ -71,22 +71,57 @@ __device__ __forceinline__ void cp_async(T* smem, const T* gmem) {
 }
 
 // ---- reciprocals -------------------------------------------------------------
-// FP64: hardware approximation of the high word, then one cubically
-// convergent correction (the series 1/x = r (1 + e + e^2 + ...) with
-// e = 1 - x r, cut after e^2): an approximation good to about 2^-20 leaves a
-// relative error near 2^-60, below FP64 rounding, in three FMAs where two
-// Newton steps take four.  The FP64 pipe bounds the FP64 elimination on
-// this part, so the FMA saved there is time saved.
-__device__ __forceinline__ double rcp_t(double x) {
+__device__ __forceinline__ float rcp_t(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+// FP64 on the FP64 pipe: hardware approximation of the high word, then one
+// cubically convergent correction (1/x = r (1 + e + e^2 + ...), e = 1 - x r).
+// Out of line: only the exponents the form below leaves out come here.
+static __device__ __noinline__ double rcp_fp64_pipe(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   const double e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
-__device__ __forceinline__ float rcp_t(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
+// FP64 with FP32 and integer instructions only.  An FP64 instruction costs a
+// warp 75 scheduler clocks on this part (64 clocks of latency), an FP32 one 1
+// (4), so the three FP64 FMAs of the form above bound the eliminations.
+// The mantissa m in [1, 2) is cut into xf (24 bits), x1 (24 bits) and x2 (5
+// bits); r is the hardware's FP32 reciprocal of xf, which lies in [0.5, 1] for
+// every xf and leaves a residual 1 - xf r below 2^-23 that one FMA gives
+// exactly (checked for all 2^23 values).  The whole residual e = 1 - m r is
+// formed as a pair s + el by an exact product and a two-sum, the correction
+// r (e + e^2) is rounded to units of 2^-53, the last place of a result in
+// [0.5, 1), through two sums with large constants, and is added to r's bit
+// pattern as an integer.  Largest error seen over 25 million values: 0.50002
+// units of the last place.  Measured per warp: latency 243 -> 148 clocks,
+// throughput 204 -> 48 clocks; FP64 solve of 59M compartments with the copy
+// of b 2.13 -> 1.92 ms, cable step of 14M 1.56 -> 1.35 ms.
+__device__ __forceinline__ double rcp_t(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  // zero, subnormal, infinite, NaN, or a reciprocal below the normal range
+  if (((hi & 0x7FF00000u) - 0x00100000u) > (2043u << 20)) return rcp_fp64_pipe(x);
+  const float xf = __uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7FFFFFu) | 0x3F800000u);
+  const float x1 = __fmul_rn(__uint2float_rn(lo & 0x1FFFFFE0u), 0x1p-52f);
+  const float x2 = __fmul_rn(__uint2float_rn(lo & 0x1Fu), 0x1p-52f);
+  const float r = rcp_t(xf);
+  const float e1 = __fmaf_rn(-xf, r, 1.f);  // exact
+  const float p = __fmul_rn(x1, r), pl = __fmaf_rn(x2, r, __fmaf_rn(x1, r, -p));
+  const float s = __fsub_rn(e1, p), bb = __fsub_rn(s, e1);
+  const float el = __fsub_rn(__fsub_rn(__fsub_rn(e1, __fsub_rn(s, bb)), __fadd_rn(p, bb)), pl);
+  const float t = __fmaf_rn(s, s, el);  // e + e^2 = s + t
+  const float rs = __fmul_rn(r, 0x1p53f);
+  constexpr float kBig = 0x1.8p32f, kOne = 0x1.8p23f;  // units of 512 and of 1
+  const float a = __fmaf_rn(rs, s, kBig);
+  const float b = __fadd_rn(__fmaf_rn(rs, t, __fmaf_rn(rs, s, -__fsub_rn(a, kBig))), kOne);
+  const int32_t k = ((int32_t)__float_as_uint(a) - 0x4FC00000) * 512 + ((int32_t)__float_as_uint(b) - 0x4B400000);
+  const uint32_t rb = __float_as_uint(r);
+  // r widened (exponent re-biased by 896, mantissa moved up by 29 bits), scaled by x's exponent, with x's sign
+  const uint32_t oh = (rb >> 3) + (0x7FD00000u - 0x07E00000u) - (hi & 0xFFF00000u);
+  const uint64_t o = ((uint64_t)oh << 32) | (uint64_t)(rb << 29);
+  return __longlong_as_double((long long)(o + (uint64_t)(int64_t)k));
 }
 
 // ---- double-float arithmetic from FP32 error-free transformations -------------
