@@ -68,6 +68,13 @@ hines_status upload(hines_plan_t p) {
     pkm[2 * k] = H.pk_blk[k];
     pkm[2 * k + 1] = H.pk_pcomp[k];
   }
+  // work entries; every chunk holds a branch, so tlvl_ptr has at most nb + n_tasks < 2^32 positions
+  std::vector<int4> phase_rec(H.phase_entry.size());
+  for (size_t k = 0; k < H.phase_entry.size(); ++k) {
+    const int32_t t = H.phase_entry[k] >> 2;
+    phase_rec[k] = make_int4((int)(uint32_t)H.task_lvl_off[(size_t)t], H.task_nlvl[(size_t)t], t,
+                             H.phase_entry[k] & 3);
+  }
   std::vector<Item> items = {
       {tmeta.data(), tmeta.size() * sizeof(hines::BrMetaT), (const void**)&D.tmeta},
       {pkm.data(), pkm.size() * 8, (const void**)&D.pk_meta},
@@ -77,7 +84,7 @@ hines_status upload(hines_plan_t p) {
       {H.task_lvl_off.data(), H.task_lvl_off.size() * 8, (const void**)&D.task_lvl_off},
       {H.tlvl_ptr.data(), H.tlvl_ptr.size() * 4, (const void**)&D.tlvl_ptr},
       {H.tchild.data(), H.tchild.size() * 4, (const void**)&D.tchild},
-      {H.phase_entry.data(), H.phase_entry.size() * 4, (const void**)&D.phase_entry},
+      {phase_rec.data(), phase_rec.size() * sizeof(int4), (const void**)&D.phase_rec},
       {H.cell_top_task.data(), H.cell_top_task.size() * 4, (const void**)&D.cell_top_task},
       {H.counter_init.data(), H.counter_init.size() * 4, (const void**)&D.counter_init},
       {H.task_sub.data(), H.task_sub.size() * 4, (const void**)&D.task_sub},
@@ -138,6 +145,8 @@ hines_status upload(hines_plan_t p) {
   D.counter = reinterpret_cast<int32_t*>(w);
   D.cell_pending = D.counter + 4;
   w += cnt_b;
+  if (cudaMemcpy(D.counter, H.counter_init.data(), H.counter_init.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess)
+    return HINES_ERR_CUDA;
   D.rw = w;
   w += rw_b;
   D.ff4 = w;

@@ -17,6 +17,13 @@ struct __align__(16) BrMetaT {
   int16_t xtask;    // 1: some child is in another task (written by another warp in the same launch)
 };
 
+// A task as the kernels run it: where its chunk boundaries start (tlvl_ptr),
+// its chunks, its number, its visits (0 both, 1 elimination, 2 substitution).
+struct TaskRec {
+  uint32_t lvl_off;
+  int32_t nlvl, id, code;
+};
+
 // Device copy of the host plan (pointers into one metadata allocation) and
 // the plan's workspace.
 struct DevPlan {
@@ -39,10 +46,10 @@ struct DevPlan {
   const int32_t* tlvl_ptr = nullptr;      // per task nlvl + 1 positions
   const BrMetaT* tmeta = nullptr;         // [nb] by position
   const int32_t* tchild = nullptr;        // child positions (non-contiguous children)
-  const int32_t* phase_entry = nullptr;   // 4 * task + visits, phases A, B (empty), C concatenated
+  const int4* phase_rec = nullptr;        // work entries, phases A, B (empty), C concatenated: the words of a TaskRec
   int32_t phase_off[4] = {0, 0, 0, 0};
   int32_t* counter = nullptr;             // [4 + n_cells] work counters, then cell_pending (workspace)
-  const int32_t* counter_init = nullptr;  // [4 + n_cells] values restored before every solve
+  const int32_t* counter_init = nullptr;  // [4 + n_cells] their values between calls (each launch restores them)
   const int32_t* cell_top_task = nullptr; // [n_cells] task of the cell's top part, -1 if not cut
   const int32_t* task_sub = nullptr;      // [2 * n_wtasks] (cell, subtree units) of a subtree task
   const int32_t* pos_branch = nullptr;    // [nb] branch id (natural numbering) of each position
