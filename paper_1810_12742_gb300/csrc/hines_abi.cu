@@ -45,22 +45,25 @@ hines_status upload(hines_plan_t p) {
   for (size_t k = 0; k < H.torder.size(); ++k) {
     const int32_t b = H.torder[k];
     hines::BrMetaT& m = tmeta[k];
-    m.first = H.br_first[(size_t)b];
-    m.len = (int16_t)H.br_len[(size_t)b];
+    const uint64_t first = (uint64_t)H.br_first[(size_t)b];  // below 2^34 (build_host_plan)
+    m.first_lo = (uint32_t)first;
+    m.first_hi_len = (uint32_t)(first >> 32) | (uint32_t)H.br_len[(size_t)b] << 24;
     const int32_t pb = H.br_parent[(size_t)b];
     m.pcomp = pb < 0 ? -1 : H.br_first[(size_t)pb] + H.br_len[(size_t)pb] - 1;
     m.ppos = pb < 0 ? -1 : H.tpos[(size_t)pb];
     const int32_t cb = H.tchild_ptr[k], ce = H.tchild_ptr[k + 1];
-    m.nchild = (int16_t)(ce - cb);
+    m.nchild = (uint16_t)(ce - cb);
     int32_t lo = INT32_MAX, hi = -1;
-    m.xtask = 0;
+    bool xtask = false;
     for (int32_t q = cb; q < ce; ++q) {
       lo = std::min(lo, H.tchild[(size_t)q]);
       hi = std::max(hi, H.tchild[(size_t)q]);
-      if (H.br_task[(size_t)H.torder[(size_t)H.tchild[(size_t)q]]] != H.br_task[(size_t)b]) m.xtask = 1;
+      xtask |= H.br_task[(size_t)H.torder[(size_t)H.tchild[(size_t)q]]] != H.br_task[(size_t)b];
     }
-    m.ccontig = (int16_t)(ce > cb && hi - lo + 1 == ce - cb);
-    m.cpos = m.ccontig ? lo : cb;
+    const bool contig = ce > cb && hi - lo + 1 == ce - cb;
+    m.child0 = contig ? lo : ce > cb ? H.tchild[(size_t)cb] : 0;
+    m.child1 = ce - cb == 2 ? (contig ? lo + 1 : H.tchild[(size_t)cb + 1]) : cb;
+    m.flags = (uint16_t)((contig ? 1 : 0) | (xtask ? 2 : 0));
   }
   // solver layout: per position (block offset, parent's solver-layout index)
   std::vector<int64_t> pkm(2 * H.torder.size());

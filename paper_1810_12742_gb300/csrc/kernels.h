@@ -7,14 +7,15 @@ namespace hines {
 
 // Per-branch metadata in task order (one entry per position of torder).
 struct __align__(16) BrMetaT {
-  int64_t first;    // natural-layout index of the proximal compartment
-  int64_t pcomp;    // natural-layout index of the parent compartment, -1 for a cell's root branch
-  int32_t ppos;     // position of the parent branch, -1 for a cell's root branch
-  int32_t cpos;     // children: first child position if contiguous, else first index into tchild
-  int16_t len;      // compartments (1..16)
-  int16_t nchild;   // children
-  int16_t ccontig;  // 1: the children are positions cpos .. cpos + nchild - 1
-  int16_t xtask;    // 1: some child is in another task (written by another warp in the same launch)
+  uint32_t first_lo;      // natural-layout index of the proximal compartment, low word
+  uint32_t first_hi_len;  // its high word (24 bits), compartments (1..16) above
+  int64_t pcomp;          // natural-layout index of the parent compartment, -1 for a cell's root branch
+  int32_t ppos;           // position of the parent branch, -1 for a cell's root branch
+  int32_t child0;         // position of the first child
+  int32_t child1;         // two children: position of the second; more: index of the first child in tchild
+  uint16_t nchild;        // children
+  uint16_t flags;         // 1: the children are positions child0 .. child0 + nchild - 1; 2: some child is in
+                          // another task (written by another warp in the same launch)
 };
 
 // A task as the kernels run it: where its chunk boundaries start (tlvl_ptr),
@@ -79,7 +80,7 @@ struct DevPlan {
 
 // One call of the warp-task kernels (unit_kernels.cuh): the mode and its arrays.
 enum class UnitOp {
-  F64, F32, F32Resolve, Comp, Cable, CableReuse, PkF64, PkF32, PkComp, PkCable, PkCableReuse,
+  F64, F32, Comp, Cable, CableReuse, PkF64, PkF32, PkComp, PkCable, PkCableReuse,
   // refinement steps on the FP32 factor (natural layout): x in FP32 or as a
   // double-float pair, x + c out as a pair or in FP64
   Refine32to2, Refine32to64, Refine2to2, Refine2to64
@@ -105,8 +106,6 @@ struct UnitCall {
 cudaError_t prepare_unit_kernels(DevPlan& P);
 cudaError_t launch_unit_solve_f64(const DevPlan& P, const double* d, const double* u, double* b, cudaStream_t s);
 cudaError_t launch_unit_solve_f32(const DevPlan& P, const float* d, const float* u, float* b, cudaStream_t s);
-// FP32 solve of a new right-hand side with the factor launch_unit_solve_f32 left in the workspace.
-cudaError_t launch_unit_resolve_f32(const DevPlan& P, const float* u, float* b, cudaStream_t s);
 cudaError_t launch_unit_solve_compensated(const DevPlan& P, const float* d, const float* u, const float* b, double* x,
                                           cudaStream_t s);
 cudaError_t launch_unit_cable(const DevPlan& P, const double* sv, const double* g, const double* u, double* V,

@@ -41,11 +41,6 @@ cudaError_t launch_unit_solve_f32(const DevPlan& P, const float* d, const float*
   c.d = d, c.u = u, c.x = b;
   return run(P, c, s);
 }
-cudaError_t launch_unit_resolve_f32(const DevPlan& P, const float* u, float* b, cudaStream_t s) {
-  UnitCall c = call(UnitOp::F32Resolve);
-  c.u = u, c.x = b;
-  return run(P, c, s);
-}
 cudaError_t launch_unit_solve_compensated(const DevPlan& P, const float* d, const float* u, const float* b, double* x,
                                           cudaStream_t s) {
   UnitCall c = call(UnitOp::Comp);

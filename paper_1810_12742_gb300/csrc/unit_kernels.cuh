@@ -80,7 +80,7 @@ struct VOf<2> {
 struct Piece {
   long long first, pcomp;  // natural: proximal compartment, parent compartment; solver layout: the chunk's
                            // block offset, the parent's solver-layout index (-1 at a cell's root)
-  int ppos, cpos, len, nchild, ccontig, xtask;
+  int ppos, child0, child1, len, nchild, ccontig, xtask;
 };
 // A parent's solution fetched ahead: a double-float pair (compensated and
 // refinement modes) or one value of the solve's type (factor modes).
@@ -102,6 +102,9 @@ struct Meta {
   // predecessor left it, fetched while the chunk is staged so that its
   // latency overlaps the staging copies
   PreX xpre[P];
+  // elimination (FP64): the contributions of the first two children, where
+  // other chunks than the cached predecessor left them, fetched likewise
+  double2 cpre[P][2];
   int L;         // rows of the lane: length of its first (longer) piece, 0 for a lane without pieces
 };
 
@@ -131,7 +134,7 @@ __device__ __forceinline__ RawMeta<kPk, P> load_meta(const DevPlan& Pl, int c0, 
   for (int h = 0; h < P; ++h) {
     const int i = P * lane + h;
     m.a[h] = make_uint4(0u, 0u, ~0u, ~0u);  // no piece: first 0, parents -1, length 0
-    m.b[h] = make_uint4(~0u, 0u, 0u, 0u);
+    m.b[h] = make_uint4(~0u, 0u, 0u, 0u);  // (no children)
     if (kPk) m.pk[h] = make_longlong2(0, -1);
     if (i < n) {
       const uint4* t = reinterpret_cast<const uint4*>(Pl.tmeta + c0 + i);
@@ -151,22 +154,28 @@ __device__ __forceinline__ Meta<P> unpack_meta(const RawMeta<kPk, P>& r) {
   for (int h = 0; h < P; ++h) {
     Piece& q = m.p[h];
     const uint4 a = r.a[h], b = r.b[h];
-    q.first = kPk ? r.pk[h].x : (long long)(((unsigned long long)a.y << 32) | a.x);
+    q.first = kPk ? r.pk[h].x : (long long)(((unsigned long long)(a.y & 0xFFFFFFu) << 32) | a.x);
     q.pcomp = kPk ? r.pk[h].y : (long long)(((unsigned long long)a.w << 32) | a.z);
     q.ppos = (int)b.x;
-    q.cpos = (int)b.y;
-    q.len = (int)(b.z & 0xFFFFu);
-    q.nchild = (int)(b.z >> 16);
-    q.ccontig = (int)(b.w & 0xFFFFu);
-    q.xtask = (int)(b.w >> 16);
+    q.child0 = (int)b.y;
+    q.child1 = (int)b.z;
+    q.len = (int)(a.y >> 24);
+    q.nchild = (int)(b.w & 0xFFFFu);
+    q.ccontig = (int)((b.w >> 16) & 1u);
+    q.xtask = (int)(b.w >> 17);
     m.xpre[h].d = 0.0;
+    m.cpre[h][0] = m.cpre[h][1] = make_double2(0.0, 0.0);
   }
   m.L = m.p[0].len;
   return m;
 }
 
+// Position of child c: the first two children of a piece with at most two are
+// in its record, so that their contributions need no dependent load.
 __device__ __forceinline__ int child_pos(const DevPlan& Pl, const Piece& q, int c) {
-  return q.ccontig ? q.cpos + c : __ldg(Pl.tchild + q.cpos + c);
+  if (c == 0) return q.child0;
+  if (q.nchild == 2) return q.child1;
+  return q.ccontig ? q.child0 + c : __ldg(Pl.tchild + q.child1 + c);
 }
 
 // A child's contribution slot: through L2 when another warp may have written
@@ -211,31 +220,46 @@ __device__ __forceinline__ void build_row_table(int L, int lane, int* tab) {
   __syncwarp();
 }
 
+// Piece i of the chunk (its owner lane's metadata, by shuffle; every lane calls it).
+struct ChunkElem {
+  long long first;
+  int len, rows;  // compartments; rows of the owner lane
+  bool root;      // holds its cell's root compartment
+};
+template <int P>
+__device__ __forceinline__ ChunkElem chunk_elem(const Meta<P>& m, int i) {
+  const int src = (i / P) & 31;
+  ChunkElem c;
+  c.first = __shfl_sync(kFull, m.p[0].first, src);
+  c.len = __shfl_sync(kFull, m.p[0].len, src);
+  int root = __shfl_sync(kFull, (int)(m.p[0].pcomp < 0), src);
+  c.rows = P == 2 ? __shfl_sync(kFull, m.L, src) : c.len;
+  if constexpr (P == 2) {
+    const long long f1 = __shfl_sync(kFull, m.p[1].first, src);
+    const int l1 = __shfl_sync(kFull, m.p[1].len, src);
+    const int r1 = __shfl_sync(kFull, (int)(m.p[1].pcomp < 0), src);
+    if (i & 1) {
+      c.first = f1;
+      c.len = l1;
+      root = r1;
+    }
+  }
+  c.root = root != 0;
+  return c;
+}
+
 // Every element of the chunk's pieces in the natural layout: sixteen lanes
-// per piece, two pieces per step (pieces are at most 16 long); the owner
-// lane's metadata comes by shuffle.  f(i, t, row, g, root) for piece i,
-// distance t from its proximal end, row of the staged chunk, natural index g,
-// and whether the piece holds its cell's root compartment (its parent is none).
+// per piece, two pieces per step (pieces are at most 16 long).  f(i, t, row,
+// g, root) for piece i, distance t from its proximal end, row of the staged
+// chunk, natural index g, and whether the piece holds its cell's root
+// compartment (its parent is none).
 template <int P, typename F>
 __device__ __forceinline__ void for_chunk_elements(const Meta<P>& m, int n, int lane, F&& f) {
   const int half = lane >> 4, t = lane & 15;
   for (int j = 0; j < n; j += 2) {
-    const int i = j + half, src = (i / P) & 31;
-    long long first = __shfl_sync(kFull, m.p[0].first, src);
-    int len = __shfl_sync(kFull, m.p[0].len, src);
-    int root = __shfl_sync(kFull, (int)(m.p[0].pcomp < 0), src);
-    const int rows = P == 2 ? __shfl_sync(kFull, m.L, src) : len;
-    if constexpr (P == 2) {
-      const long long f1 = __shfl_sync(kFull, m.p[1].first, src);
-      const int l1 = __shfl_sync(kFull, m.p[1].len, src);
-      const int r1 = __shfl_sync(kFull, (int)(m.p[1].pcomp < 0), src);
-      if (i & 1) {
-        first = f1;
-        len = l1;
-        root = r1;
-      }
-    }
-    if (i < n && t < len) f(i, t, rows - 1 - t, first + t, root != 0);
+    const int i = j + half;
+    const ChunkElem c = chunk_elem(m, i);
+    if (i < n && t < c.len) f(i, t, c.rows - 1 - t, c.first + t, c.root);
   }
 }
 
@@ -345,6 +369,10 @@ struct CompMode {
   static constexpr bool kPacked = kPk;
   static constexpr bool kNeedsBlk = true;
   static constexpr int kPer = P;
+  // row loops: the natural layout's longer chunk code does better in fewer
+  // copies (28M compartments 833 against 891 us), the solver layout's does not
+  // (21M with the unpack 836 against 827 us)
+  static constexpr int kUnroll = kPk ? kL : 4;
   struct Args {
     const float* d;
     const float* u;
@@ -463,7 +491,7 @@ struct CompMode {
       }
       FFV<V> D{vpack<P>(d0h), vpack<P>(d0l)}, B{vpack<P>(b0h), vpack<P>(b0l)};
       // row r: g = u / D, y = B / D into the factor block; then the chain to row r + 1
-#pragma unroll
+#pragma unroll kUnroll
       for (int r = 0; r < kL - 1; ++r) {
         if (r < L - 1) {
           const V uk = ldv(su, rows.slot(r, me), V{});
@@ -522,7 +550,7 @@ struct CompMode {
     }
     FFV<V> X{vpack<P>(xph), vpack<P>(xpl)};
     float xbh = 0.f, xbl = 0.f;  // the second piece's distal solution
-#pragma unroll
+#pragma unroll kUnroll
     for (int r = kL - 1; r >= 0; --r) {
       if (r < L) {
         const int q = tab[r] + me;
@@ -573,25 +601,39 @@ struct CompMode {
 };
 
 // ============================================================================
-// Factor mode (FP64, FP32, passive cable): the elimination leaves, per
-// compartment, the reciprocal eliminated diagonal and the eliminated
-// right-hand side; the substitution reads them back.  FP64 writes the pair
-// as 16 bytes into the plan's factor block, in the chunk's block order of the
-// solver layout (each row a contiguous run), and the substitution stages it
-// with bulk copies in either layout; FP32 writes the reciprocal to the
-// workspace at natural positions and the right-hand side in place (the
-// refinement reads that factor).  In cable mode
+// Factor mode (FP64, FP32, passive cable).  FP64: the elimination leaves, per
+// compartment, g = u / D and y = B / D (D, B: the eliminated pivot and
+// right-hand side), and the substitution runs x = y - g x_parent: one FP64
+// instruction a row, no input read again.  The pair goes either into the
+// plan's factor block, 16 bytes in the chunk's block order of the solver
+// layout (each row a contiguous run), staged back with bulk copies, or to
+// natural (or slot) positions, g into the workspace and y in place.  A full
+// cable step also leaves the reciprocal pivot, which steps that re-use the
+// factor need for y.  FP32: the reciprocal pivot goes to the workspace and the
+// right-hand side in place (the refinement reads that factor); the
+// substitution reads them and u back.  In cable mode
 // the system is rebuilt while staging (Section 1's implicit-Euler system):
 // d_i = s_i (1 + theta dt g_i) + sum of a over the edges at i (a = -u),
 // b_i = s_i V_i + s_i dt g_i (E - (1 - theta) V_i).
 // The lane's pieces are handled one after the other in the same loop step
 // (no packed FP64 instructions exist), their rows aligned as in the compensated
 // mode; a piece's rows before its distal row are skipped.
+//
+// The cable matrix is eliminated without its subtractions: with
+// E_i = s_i (1 + theta dt g_i) + sum over the children c of a_c E_c / D_c, the
+// conductance to ground seen at i, the pivot is D_i = E_i + a_i (a cell's
+// root: E_i), since a_c - a_c^2 / D_c = a_c E_c / D_c.  The same number of
+// operations, and nothing cancels where the leak is small next to a.
+//
+// The FP64 pipe and the latency of a row bound this mode: an FP64 instruction
+// takes 75 scheduler clocks per warp (64 clocks of latency), so a row holds as
+// few of them as possible (elimination 4, cable 5, substitution 1), and the
+// next row's inputs are read before the current row's results are written
+// (the compiler may not move them over the stores).
 // ============================================================================
-// kReuse: the elimination of a new right-hand side with the factor a previous
-// solve of the same plan and matrix left in the workspace (the reciprocal
-// eliminated diagonal): only b is eliminated (the refinement's correction
-// solves; passive-cable steps after the first, the matrix being constant).
+// kReuse: a passive-cable step with the factor a full step of the same plan
+// and matrix left in the workspace: only the right-hand side is rebuilt and
+// eliminated.
 // kBlk: FP64 keeps its factor in block order (else at natural positions, as
 // FP32 always does).
 template <typename T, bool kCable, bool kPk, int P, bool kReuse = false, bool kBlk = true>
@@ -607,9 +649,16 @@ struct FactorMode {
     return r;
   }
   static constexpr bool kPacked = kPk;
-  static constexpr bool kBF = kBlk && sizeof(T) == 8;  // the factor in block order (FP64)
+  static constexpr bool kYG = sizeof(T) == 8;  // the factor is (g, y)
+  static constexpr bool kBF = kBlk && kYG;     // ... in block order
   static constexpr bool kNeedsBlk = kBF;
   static constexpr int kPer = P;
+  // row loops: sixteen copies of the long FP64 row overrun the instruction
+  // cache (4 against 16: 64 small cells 47.1 against 51.2 us, 59M compartments
+  // 1.60 against 1.65 ms); a row that re-uses its factor is short (7.65
+  // against 7.29 ms per 40 steps of 1.7M compartments)
+  static constexpr int kUnroll = kYG && !kReuse ? 4 : kL;
+  static_assert(!kReuse || (kCable && kYG), "only FP64 cable steps re-use a factor");
   struct Args {
     const T* d;
     const T* u;
@@ -617,7 +666,7 @@ struct FactorMode {
     const T* g;
     T* x;        // right-hand side in, solution out (cable: V in, V out)
     T dt, E, theta;
-    bool rhs_from_V;
+    bool rhs_from_V;  // cable: a time step (else a solve with the step's matrix, which leaves no reciprocals)
     const T* rhs = nullptr;  // non-null: the right-hand side is read from here (x receives the solution)
   };
   // a staging buffer: d (or the factor), u, b, then the row table (solver layout)
@@ -638,27 +687,91 @@ struct FactorMode {
   __device__ static void init_warp(unsigned char* wbase, int lane) {
     if (kBulk) Bulk::init(wbase, lane);
   }
+  // (g, y) per slot of the solver layout
   __device__ static double2* factor_block(const DevPlan& Pl) { return static_cast<double2*>(Pl.ff4); }
+  // the reciprocal pivots of the last full step: the workspace the other placement's factor would use
+  __device__ static T* reciprocals(const DevPlan& Pl) { return static_cast<T*>(kBF ? Pl.fac : Pl.ff4); }
+  __device__ static bool keeps_rcp(const Args& A) { return kYG && kCable && !kReuse && A.rhs_from_V; }
 
-  // Section 1's implicit-Euler system, each part in the fewest operations:
-  // the diagonal less the compartment's own edge to its parent,
-  // s (1 + theta dt g) - a_own, in one FMA (a cell's root, which has no such
-  // edge, adds its u back: the same operations in both layouts), and the
-  // right-hand side s (V + dt g (E - (1 - theta) V)) (theta = 1: s (V + dt E g))
-  __device__ static T cable_diag_edge(const Args& A, T si, T gi, T ui) {
-    return fma(si, fma(A.theta * A.dt, gi, T(1)), -ui);
-  }
+  // Section 1's implicit-Euler system, each part in the fewest operations: the
+  // diagonal less all its edges, s (1 + theta dt g), and the right-hand side
+  // s (V + dt g (E - (1 - theta) V)) (theta = 1: s (V + dt E g))
+  __device__ static T cable_diag(const Args& A, T si, T gi) { return si * fma(A.theta * A.dt, gi, T(1)); }
   __device__ static T cable_rhs(const Args& A, T si, T gi, T vi) {
     if (A.theta == T(1)) return si * fma(A.dt * A.E, gi, vi);
     return si * fma(A.dt * gi, fma(A.theta - T(1), vi, A.E), vi);
   }
+
+  // Rebuild of the chunk's system (cable, elimination).  kStep elements per
+  // lane are loaded before any is computed: one at a time, every element
+  // waited for its loads (19.6k clocks a chunk of the 15M-compartment step,
+  // more than the elimination itself).
+  static constexpr int kStep = kReuse ? 4 : 2;
+  struct Elem {
+    T s, g, u, v;
+    __device__ void load(const Args& A, long long i) {
+      v = A.x[i];
+      if (!kReuse) u = A.u[i];
+      if (!kReuse || A.rhs_from_V) {
+        s = A.s[i];
+        g = A.g[i];
+      }
+    }
+    __device__ void store(const Args& A, T* sd, T* su, T* sb, int q) const {
+      if (!kReuse) {
+        sd[q] = cable_diag(A, s, g);
+        su[q] = u;
+      }
+      sb[q] = A.rhs_from_V ? cable_rhs(A, s, g, v) : v;
+    }
+  };
+  __device__ static void rebuild_block(const Args& A, long long blk, int e, int lane, T* sd, T* su, T* sb) {
+    for (int i0 = lane; i0 < e; i0 += 32 * kStep) {
+      Elem el[kStep];
+#pragma unroll
+      for (int k = 0; k < kStep; ++k)
+        if (i0 + 32 * k < e) el[k].load(A, blk + i0 + 32 * k);
+#pragma unroll
+      for (int k = 0; k < kStep; ++k)
+        if (i0 + 32 * k < e) el[k].store(A, sd, su, sb, i0 + 32 * k);
+    }
+  }
+  template <typename F>
+  __device__ static void rebuild_natural(const Args& A, const Meta<P>& m, int n, int lane, T* sd, T* su, T* sb, F&& f) {
+    const int half = lane >> 4, t = lane & 15;
+    for (int j = 0; j < n; j += 2 * kStep) {
+      Elem el[kStep];
+      int q[kStep];  // word of the staged chunk, -1: none
+#pragma unroll
+      for (int k = 0; k < kStep; ++k) {
+        const int i = j + 2 * k + half;
+        const ChunkElem c = chunk_elem(m, i);
+        q[k] = i < n && t < c.len ? nidx<P>(c.rows - 1 - t, i) : -1;
+        if (q[k] >= 0) {
+          el[k].load(A, c.first + t);
+          f(i, c.rows - 1 - t, q[k], c.first + t);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < kStep; ++k)
+        if (q[k] >= 0) el[k].store(A, sd, su, sb, q[k]);
+    }
+  }
+
+  // A child's contribution (D, B): from the cache of the chunk just before,
+  // or from the slots.
+  __device__ static bool local_child(int cp, const Prev& pv) { return cp >= pv.c0 && cp < pv.c0 + pv.n; }
 
   __device__ static void stage(const DevPlan& Pl, const Args& A, int visit, Meta<P>& m, int n, int lane,
                                unsigned char* buf, const Prev& pv) {
     T* sd = reinterpret_cast<T*>(buf);
     T* su = sd + G::kSlots;
     T* sb = su + G::kSlots;
-    const T* fac = static_cast<const T*>(Pl.fac);
+    int* tab = reinterpret_cast<int*>(buf + kTab);
+    T* fac = static_cast<T*>(Pl.fac);
+    if (kBF || kPk) build_row_table<P>(m.L, lane, tab);
+    const int e = (kBF || kPk) ? tab[kL] : 0;
+    const long long blk = kPk ? __shfl_sync(kFull, m.p[0].first, 0) : 0;
     if (visit == 1) {
       // the parent's solution, unless the predecessor chunk's cache holds it
       // (a chunk staged before its predecessor is computed finds that
@@ -669,112 +782,76 @@ struct FactorMode {
         const int loc = q.ppos - pv.c0;
         if (q.len > 0 && q.pcomp >= 0 && !(loc >= 0 && loc < pv.n)) pre_set(m.xpre[h], A.x[q.pcomp]);
       }
-    }
-    if constexpr (kBF) {
-      int* tab = reinterpret_cast<int*>(buf + kTab);
-      build_row_table<P>(m.L, lane, tab);
-      const int e = tab[kL];
-      const long long blk = kPk ? __shfl_sync(kFull, m.p[0].first, 0) : 0;
-      if (visit == 1) {
-        // the factor block (reciprocal pivot, eliminated right-hand side) over
-        // the first two arrays, u in the third
+      if constexpr (kBF) {  // the factor block over the first two arrays
         Bulk::template issue<1>(buf, lane, (unsigned)e * 16u, buf, factor_block(Pl) + m.blk);
-        if (kPk) {
-          stage_block(sb, A.u, blk, e, lane);
-        } else {
-          for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
-            cp_async(&sb[nidx<P>(row, i)], A.u + g);
-          });
-        }
+      } else if (kPk) {
+        stage_block(sd, static_cast<const T*>(fac), blk, e, lane);
+        if (!kYG) stage_block(su, A.u, blk, e, lane);
+        stage_block(sb, static_cast<const T*>(A.x), blk, e, lane);
         cp_commit();
-        return;
-      }
-      if (kReuse) {
-        // the stored reciprocal pivots from the block, u, and b rebuilt
-        const double* rp = reinterpret_cast<const double*>(factor_block(Pl) + m.blk);
-        if (kPk) {
-          for (int i = lane; i < e; i += 32) cp_async(&sd[i], rp + 2 * i);
-          stage_block(su, A.u, blk, e, lane);
-          for (int i = lane; i < e; i += 32) {
-            const long long g = blk + i;
-            const T vi = A.x[g];
-            sb[i] = A.rhs_from_V ? cable_rhs(A, A.s[g], A.g[g], vi) : vi;
-          }
-        } else {
-          for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
-            const int q = nidx<P>(row, i);
-            cp_async(&sd[q], rp + 2 * (tab[row] + i));
-            cp_async(&su[q], A.u + g);
-            const T vi = A.x[g];
-            sb[q] = A.rhs_from_V ? cable_rhs(A, A.s[g], A.g[g], vi) : vi;
-          });
-        }
-        cp_commit();
-        return;
-      }
-    }
-    if (kPk) {
-      int* tab = reinterpret_cast<int*>(buf + kTab);
-      if constexpr (!kBF) build_row_table<P>(m.L, lane, tab);
-      const long long blk = __shfl_sync(kFull, m.p[0].first, 0);
-      const int e = tab[kL];
-      if (kCable && visit == 0) {
-        // the block's rows in place; every diagonal loses its own edge here,
-        // and compute() gives it back to a cell's root compartment (known there)
-        if (kReuse) {  // the stored factor; only the right-hand side is rebuilt
-          stage_block(sd, fac, blk, e, lane);
-          stage_block(su, A.u, blk, e, lane);
-        }
-        for (int i = lane; i < e; i += 32) {
-          const long long g = blk + i;
-          const T vi = A.x[g];
-          if (kReuse) {
-            sb[i] = A.rhs_from_V ? cable_rhs(A, A.s[g], A.g[g], vi) : vi;
-          } else {
-            const T si = A.s[g], gi = A.g[g], ui = A.u[g];
-            sd[i] = cable_diag_edge(A, si, gi, ui);
-            su[i] = ui;
-            sb[i] = A.rhs_from_V ? cable_rhs(A, si, gi, vi) : vi;
-          }
-        }
       } else {
-        stage_block(sd, (visit == 1 || kReuse) ? fac : A.d, blk, e, lane);
-        stage_block(su, A.u, blk, e, lane);
-        stage_block(sb, (visit == 0 && A.rhs) ? A.rhs : static_cast<const T*>(A.x), blk, e, lane);
+        for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
+          const int q = nidx<P>(row, i);
+          cp_async(&sd[q], fac + g);
+          if (!kYG) cp_async(&su[q], A.u + g);
+          cp_async(&sb[q], static_cast<const T*>(A.x) + g);
+        });
+        cp_commit();
       }
-      cp_commit();
       return;
     }
-    if (visit == 1 || !kCable) {
-      const T* dsrc = (visit == 1 || kReuse) ? fac : A.d;
-      const T* bsrc = (visit == 0 && A.rhs) ? A.rhs : A.x;
-      for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
-        const int q = nidx<P>(row, i);
-        cp_async(&sd[q], dsrc + g);
-        cp_async(&su[q], A.u + g);
-        cp_async(&sb[q], bsrc + g);
-      });
-    } else if (kReuse) {  // cable, stored factor: only the right-hand side is rebuilt
-      for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
-        const int q = nidx<P>(row, i);
-        cp_async(&sd[q], fac + g);
-        cp_async(&su[q], A.u + g);
-        const T vi = A.x[g];
-        sb[q] = A.rhs_from_V ? cable_rhs(A, A.s[g], A.g[g], vi) : vi;
-      });
+    if constexpr (kReuse) {
+      // the stored reciprocals and g, and the right-hand side rebuilt
+      const T* rc = reciprocals(Pl);
+      const T* gp = kBF ? reinterpret_cast<const T*>(factor_block(Pl) + m.blk) : fac;  // g: every other word, or by index
+      if (kPk) {
+        stage_block(sd, rc, blk, e, lane);
+        if (kBF)
+          for (int i = lane; i < e; i += 32) cp_async(&su[i], gp + 2 * i);
+        else
+          stage_block(su, gp, blk, e, lane);
+        rebuild_block(A, blk, e, lane, sd, su, sb);
+      } else {
+        rebuild_natural(A, m, n, lane, sd, su, sb, [&](int i, int row, int q, long long g) {
+          cp_async(&sd[q], kBF ? rc + m.blk + tab[row] + i : rc + g);
+          cp_async(&su[q], kBF ? gp + 2 * (tab[row] + i) : gp + g);
+        });
+      }
+    } else if constexpr (kCable) {
+      if (kPk)
+        rebuild_block(A, blk, e, lane, sd, su, sb);
+      else
+        rebuild_natural(A, m, n, lane, sd, su, sb, [](int, int, int, long long) {});
     } else {
-      // the own edge to the parent comes off every diagonal but a cell root's
-      for_chunk_elements(m, n, lane, [&](int i, int t, int row, long long g, bool root) {
-        const T si = A.s[g], gi = A.g[g], ui = A.u[g], vi = A.x[g];
-        T dd = cable_diag_edge(A, si, gi, ui);
-        if (root && t == 0) dd += ui;  // a cell's root: no edge to a parent
-        const int q = nidx<P>(row, i);
-        sd[q] = dd;
-        su[q] = ui;
-        sb[q] = A.rhs_from_V ? cable_rhs(A, si, gi, vi) : vi;
-      });
+      const T* bsrc = A.rhs ? A.rhs : static_cast<const T*>(A.x);
+      if (kPk) {
+        stage_block(sd, A.d, blk, e, lane);
+        stage_block(su, A.u, blk, e, lane);
+        stage_block(sb, bsrc, blk, e, lane);
+      } else {
+        for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
+          const int q = nidx<P>(row, i);
+          cp_async(&sd[q], A.d + g);
+          cp_async(&su[q], A.u + g);
+          cp_async(&sb[q], bsrc + g);
+        });
+      }
     }
     cp_commit();
+    if constexpr (kYG) {
+      // contributions that no cache holds are on their way with the inputs
+      const double2* slot = static_cast<const double2*>(Pl.cd);
+#pragma unroll
+      for (int h = 0; h < P; ++h) {
+        const Piece& q = m.p[h];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          if (c >= q.nchild) continue;
+          const int cp = child_pos(Pl, q, c);
+          if (!local_child(cp, pv)) m.cpre[h][c] = slot_load(slot + cp, q);
+        }
+      }
+    }
   }
 
   __device__ static void compute(const DevPlan& Pl, const Args& A, int visit, int c0, int n, int lane,
@@ -796,92 +873,102 @@ struct FactorMode {
 #pragma unroll
     for (int h = 0; h < P; ++h) first_row[h] = m.p[h].len > 0 ? L - m.p[h].len : kL;
     if (visit == 0) {
-      if (kPk && kCable && !kReuse) {
-        // solver layout: a cell's root compartment (the proximal compartment
-        // of a root piece, row L - 1) gets back the edge staging took off
-#pragma unroll
-        for (int h = 0; h < P; ++h) {
-          if (m.p[h].len > 0 && m.p[h].pcomp < 0) {
-            const int i = rows.slot(L - 1, me + h);
-            sd[i] += su[i];
-          }
-        }
-      }
-      T D[P], B[P];
+      const bool keep_rcp = keeps_rcp(A);
+      T* rcp_block = kBF ? reciprocals(Pl) + m.blk : nullptr;
+      // per piece: the eliminated pivot (cable: E) and right-hand side of the
+      // current row, its coupling (re-using a factor: its g) and stored
+      // reciprocal
+      T D[P], B[P], uk[P], rk[P];
 #pragma unroll
       for (int h = 0; h < P; ++h) {
         const Piece& q = m.p[h];
         D[h] = T(1);
-        B[h] = T(0);
+        B[h] = uk[h] = rk[h] = T(0);
         if (q.len == 0) continue;
         const int idx = rows.slot(first_row[h], me + h);
-        if (!kReuse) D[h] = sd[idx];
+        (kReuse ? rk[h] : D[h]) = sd[idx];
         B[h] = sb[idx];
-        for (int c = 0; c < q.nchild; ++c) {
+        uk[h] = su[idx];
+        auto child = [&](int c, double2 pre, bool fetched) {
           const int cp = child_pos(Pl, q, c);
-          const int loc = cp - pv.c0;
-          const bool local = loc >= 0 && loc < pv.n;
-          if (!kReuse) D[h] -= local ? cslot[(pv.which * G::kChunk + loc) * 2] : slot_load(slot + 2 * cp, q);
-          B[h] -= local ? cslot[(pv.which * G::kChunk + loc) * 2 + 1] : slot_load(slot + 2 * cp + 1, q);
+          const int w = (pv.which * G::kChunk + cp - pv.c0) * 2;
+          T cd, cb;
+          if (local_child(cp, pv)) {
+            cd = kReuse ? T(0) : cslot[w];
+            cb = cslot[w + 1];
+          } else if (fetched) {
+            cd = (T)pre.x;
+            cb = (T)pre.y;
+          } else {
+            cd = kReuse ? T(0) : slot_load(slot + 2 * (size_t)cp, q);
+            cb = slot_load(slot + 2 * (size_t)cp + 1, q);
+          }
+          if (!kReuse) D[h] -= cd;
+          B[h] -= cb;
+        };
+        int c = 0;
+        if (kYG) {
+          if (q.nchild > 0) child(0, m.cpre[h][0], true);
+          if (q.nchild > 1) child(1, m.cpre[h][1], true);
+          c = 2;
         }
+        for (; c < q.nchild; ++c) child(c, make_double2(0.0, 0.0), false);
       }
-      // rows from the distal end: store the reciprocal pivot (or, reusing the
-      // factor, read it) and the eliminated right-hand side, then pass the
-      // chain on; at the proximal row leave the contribution to the parent
-#pragma unroll
+      // one row's factor from its pivot: g (or the multiplier) is returned
+      auto factor_row = [&](int h, int r, bool root) {
+        const int i = rows.slot(r, me + h);
+        const T rr = kReuse ? rk[h] : rcp_solve(kCable && !root ? D[h] - uk[h] : D[h]);
+        const T f = kReuse ? uk[h] : uk[h] * rr;
+        if constexpr (kYG) {
+          const T y = B[h] * rr;
+          const T gs = root ? T(0) : f;  // a cell's root: x = y
+          if constexpr (kBF) {
+            const int q = tab[r] + me + h;
+            if (kReuse)
+              bf[q].y = y;
+            else
+              bf[q] = make_double2(gs, y);
+            if (keep_rcp) rcp_block[q] = rr;
+          } else {
+            if (!kReuse) sd[i] = gs;
+            if (keep_rcp) su[i] = rr;
+            sb[i] = y;
+          }
+        } else {
+          sd[i] = rr;
+          sb[i] = root ? B[h] * rr : B[h];  // a root's x
+        }
+        return f;
+      };
+      // rows from the distal end: the factor, then the chain to the next row
+#pragma unroll kUnroll
       for (int r = 0; r < kL - 1; ++r) {
         if (r < L - 1) {
-          const int i = rows.slot(r, me);
 #pragma unroll
           for (int h = 0; h < P; ++h) {
             if (r < first_row[h]) continue;
-            const T uk = su[i + h];
-            const T rr = kReuse ? sd[i + h] : rcp_solve(D[h]);
-            if constexpr (kBF) {
-              bf[tab[r] + me + h] = make_double2(rr, B[h]);
-            } else {
-              if (!kReuse) sd[i + h] = rr;
-              sb[i + h] = B[h];
-            }
-            const T f = uk * rr;
             const int i1 = rows.slot(r + 1, me + h);
-            if (!kReuse) {
-              D[h] = sd[i1] - f * uk;
-              if (kCable) D[h] -= uk;  // the edge to the chain child
-            }
-            B[h] = sb[i1] - f * B[h];
+            const T a1 = sd[i1], b1 = sb[i1], u1 = su[i1];
+            const T f = factor_row(h, r, false);
+            if (!kReuse) D[h] = a1 - f * (kCable ? D[h] : uk[h]);
+            B[h] = b1 - f * B[h];
+            uk[h] = u1;
+            rk[h] = a1;
           }
         }
       }
-      T c0v[P], c1v[P];
-      {
-        const int i = rows.slot(L - 1, me);
-#pragma unroll
-        for (int h = 0; h < P; ++h) {
-          c0v[h] = c1v[h] = T(0);
-          if (m.p[h].len == 0) continue;
-          const T uk = su[i + h];
-          const T rr = kReuse ? sd[i + h] : rcp_solve(D[h]);
-          if constexpr (kBF) bf[tab[L - 1] + me + h] = make_double2(rr, B[h]);  // a root's x is B rr
-          else if (!kReuse) sd[i + h] = rr;
-          if (m.p[h].pcomp >= 0) {
-            const T f = uk * rr;
-            if constexpr (!kBF) sb[i + h] = B[h];
-            c0v[h] = kReuse ? T(0) : (kCable ? f * uk + uk : f * uk);
-            c1v[h] = f * B[h];
-          } else if constexpr (!kBF) {
-            sb[i + h] = B[h] * rr;  // solve root
-          }
-        }
-      }
+      // the proximal row, and the contribution to the parent
 #pragma unroll
       for (int h = 0; h < P; ++h) {
         if (m.p[h].len == 0) continue;
-        const int pos = c0 + me + h;
-        slot[2 * pos] = c0v[h];
-        slot[2 * pos + 1] = c1v[h];
-        cslot[(cur * G::kChunk + me + h) * 2] = c0v[h];
-        cslot[(cur * G::kChunk + me + h) * 2 + 1] = c1v[h];
+        const bool root = m.p[h].pcomp < 0;
+        const T f = factor_row(h, L - 1, root);
+        const T cd = root || kReuse ? T(0) : f * (kCable ? D[h] : uk[h]), cb = root ? T(0) : f * B[h];
+        const size_t pos = (size_t)(c0 + me + h);
+        slot[2 * pos] = cd;
+        slot[2 * pos + 1] = cb;
+        cslot[(cur * G::kChunk + me + h) * 2] = cd;
+        cslot[(cur * G::kChunk + me + h) * 2 + 1] = cb;
       }
       return;
     }
@@ -895,27 +982,37 @@ struct FactorMode {
         xp[h] = (loc >= 0 && loc < pv.n) ? cx[pv.which * G::kChunk + loc] : pre_get(m.xpre[h], T{});
       }
     }
-    if constexpr (kBF) {
-      // the staged block: (reciprocal pivot, eliminated right-hand side) per
-      // slot in block order, u in the third array; x goes over the pivot
+    if constexpr (kYG) {
+      // x = y - g x_parent; x goes over g (block order) or over y
       const double2* fb = reinterpret_cast<const double2*>(buf);
       double* sx = reinterpret_cast<double*>(buf);
+      auto load = [&](int r, int h) {
+        if constexpr (kBF) return fb[tab[r] + me + h];
+        const int i = rows.slot(r, me + h);
+        return make_double2(sd[i], sb[i]);
+      };
+      double2 f[P];
 #pragma unroll
+      for (int h = 0; h < P; ++h) f[h] = load(L - 1, h);
+#pragma unroll kUnroll
       for (int r = kL - 1; r >= 0; --r) {
         if (r < L) {
-          const int i = rows.slot(r, me), q = tab[r] + me;
 #pragma unroll
           for (int h = 0; h < P; ++h) {
             if (r < first_row[h]) continue;
-            const double2 f = fb[q + h];
-            const T xi = (m.p[h].pcomp < 0 && r == L - 1) ? f.y * f.x : (f.y - sb[i + h] * xp[h]) * f.x;
-            sx[2 * (q + h)] = xi;
+            const double2 fk = f[h];
+            if (r > 0) f[h] = load(r - 1, h);  // (before this row's store)
+            const T xi = fk.y - fk.x * xp[h];
+            if constexpr (kBF)
+              sx[2 * (tab[r] + me + h)] = xi;
+            else
+              sb[rows.slot(r, me + h)] = xi;
             xp[h] = xi;
           }
         }
       }
     } else {
-#pragma unroll
+#pragma unroll kUnroll
       for (int r = kL - 1; r >= 0; --r) {
         if (r < L) {
           const int i = rows.slot(r, me);
@@ -937,36 +1034,40 @@ struct FactorMode {
   __device__ static void copy_out(const DevPlan& Pl, const Args& A, int visit, const Meta<P>& m, int n, int lane,
                                   unsigned char* buf) {
     const T* sd = reinterpret_cast<const T*>(buf);
-    const T* sb = sd + 2 * G::kSlots;
-    T* fac = static_cast<T*>(Pl.fac);
+    const T* su = sd + G::kSlots;
+    const T* sb = su + G::kSlots;
+    const int* tab = reinterpret_cast<const int*>(buf + kTab);
+    const long long blk = kPk ? __shfl_sync(kFull, m.p[0].first, 0) : 0;
     if constexpr (kBF) {
       // the elimination wrote its factor block directly; the substitution
-      // left x over each slot's pivot
+      // left x over each slot's g
       if (visit == 0) return;
       const double* sx = reinterpret_cast<const double*>(buf);
-      const int* tab = reinterpret_cast<const int*>(buf + kTab);
       if (kPk) {
-        const long long blk = __shfl_sync(kFull, m.p[0].first, 0);
         const int e = tab[kL];
         for (int s = lane; s < e; s += 32) A.x[blk + s] = sx[2 * s];
-        return;
+      } else {
+        for_chunk_elements(m, n, lane,
+                           [&](int i, int, int row, long long g, bool) { A.x[g] = sx[2 * (tab[row] + i)]; });
       }
-      for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) { A.x[g] = sx[2 * (tab[row] + i)]; });
       return;
     }
+    T* fac = static_cast<T*>(Pl.fac);
+    T* rc = reciprocals(Pl);
+    const bool keep_fac = visit == 0 && !kReuse, keep_rcp = visit == 0 && keeps_rcp(A);
     if (kPk) {
-      const int* tab = reinterpret_cast<const int*>(buf + kTab);
-      const long long blk = __shfl_sync(kFull, m.p[0].first, 0);
       const int e = tab[kL];
       for (int s = lane; s < e; s += 32) {
-        if (visit == 0 && !kReuse) fac[blk + s] = sd[s];
+        if (keep_fac) fac[blk + s] = sd[s];
+        if (keep_rcp) rc[blk + s] = su[s];
         A.x[blk + s] = sb[s];
       }
       return;
     }
     for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
       const int q = nidx<P>(row, i);
-      if (visit == 0 && !kReuse) fac[g] = sd[q];
+      if (keep_fac) fac[g] = sd[q];
+      if (keep_rcp) rc[g] = su[q];
       A.x[g] = sb[q];
     });
   }
@@ -1423,7 +1524,6 @@ struct UnitKernels {
   using PkF32 = FactorMode<float, false, true, PL>;
   using PkComp = CompMode<true, PL>;
   using PkCable = FactorMode<double, true, true, PL>;
-  using F32Reuse = FactorMode<float, false, false, PL, true>;
   using CableReuse = FactorMode<double, true, false, PL, true>;
   using PkCableReuse = FactorMode<double, true, true, PL, true>;
   // the FP64 kinds with the factor at natural positions (small batches)
@@ -1448,7 +1548,6 @@ struct UnitKernels {
     if (e == cudaSuccess) e = grid_of<PkComp>(P, &P.grid[6]);
     if (e == cudaSuccess) e = grid_of<PkCable>(P, &P.grid[7]);
     int g_reuse = 0;  // same footprint as the plain modes
-    if (e == cudaSuccess) e = grid_of<F32Reuse>(P, &g_reuse);
     if (e == cudaSuccess) e = grid_of<CableReuse>(P, &g_reuse);
     if (e == cudaSuccess) e = grid_of<PkCableReuse>(P, &g_reuse);
     if (e == cudaSuccess) e = grid_of<R32to2>(P, &P.grid_refine);
@@ -1483,8 +1582,6 @@ struct UnitKernels {
       case UnitOp::F32:
         return launch_phases<F32>(P, {d4, u4, nullptr, nullptr, x4, 0.f, 0.f, 0.f, false,
                                       static_cast<const float*>(c.rhs)}, P.grid[1], s);
-      case UnitOp::F32Resolve:
-        return launch_phases<F32Reuse>(P, {nullptr, u4, nullptr, nullptr, x4, 0.f, 0.f, 0.f, false}, P.grid[1], s);
       case UnitOp::Comp:
         return launch_phases<Comp>(P, {d4, u4, b4, x8}, P.grid[3], s);
       case UnitOp::Cable:
