@@ -78,7 +78,15 @@ hines_status upload(hines_plan_t p) {
     phase_rec[k] = make_int4((int)(uint32_t)H.task_lvl_off[(size_t)t], H.task_nlvl[(size_t)t], t,
                              H.phase_entry[k] & 3);
   }
+  // every task's chunks, one after the other (positions run on from task to task)
+  std::vector<int32_t> chunk_pos;
+  for (int32_t t = 0; t < H.n_tasks; ++t)
+    for (int32_t l = 0; l < H.task_nlvl[(size_t)t]; ++l)
+      chunk_pos.push_back(H.tlvl_ptr[(size_t)(H.task_lvl_off[(size_t)t] + l)]);
+  D.n_chunks = (int32_t)chunk_pos.size();
+  chunk_pos.push_back((int32_t)H.torder.size());
   std::vector<Item> items = {
+      {chunk_pos.data(), chunk_pos.size() * 4, (const void**)&D.chunk_pos},
       {tmeta.data(), tmeta.size() * sizeof(hines::BrMetaT), (const void**)&D.tmeta},
       {pkm.data(), pkm.size() * 8, (const void**)&D.pk_meta},
       {H.pk_perm.data(), H.pk_perm.size() * 8, (const void**)&D.pk_perm},

@@ -57,15 +57,18 @@ struct DevPlan {
   int32_t* cell_pending = nullptr;        // counter + 4: subtree units whose elimination is still to finish
   // solver layout (Section 5's interleaving per chunk)
   int64_t n_packed = 0;
+  int32_t n_chunks = 0;
+  const int32_t* chunk_pos = nullptr;     // [n_chunks + 1] first position of each chunk of the batch
   const longlong2* pk_meta = nullptr;     // [nb] per position: (chunk block offset, parent's solver-layout index)
   const int64_t* pk_perm = nullptr;       // [n_packed] natural index of each solver-layout slot, -1 for padding
   const int64_t* pk_edge = nullptr;       // [n_packed] natural index of each slot's coupling (pk_perm unless re-rooted)
-  int32_t grid[8] = {1, 1, 1, 1, 1, 1, 1, 1};  // persistent grid size per kernel kind
-  int32_t grid_nf[4] = {1, 1, 1, 1};           // the same for the FP64 kinds keeping the factor at natural positions
+  // persistent grid sizes per kernel kind: teams of two warps (x), CTAs of two warps with a task each (y)
+  int2 grid[8] = {};
+  int2 grid_nf[4] = {};                        // the same for the FP64 kinds keeping the factor at natural positions
   int32_t fp64_blocks = 0;                     // 1: FP64 factors in block order (hines_plan_opts.fp64_factor)
   int32_t sms = 1;                             // multiprocessors of the plan's device
   int32_t per_lane = 2;                        // branch pieces per warp lane (the plan's lane mapping)
-  int32_t grid_refine = 1;                     // persistent grid size of the refinement steps
+  int2 grid_refine = {};                       // the same for the refinement steps
   // workspace
   void* fac = nullptr;    // 8 bytes per natural or solver-layout slot: factor (FP64 / FP32 solves), FP32 working
                           // arrays (refine)

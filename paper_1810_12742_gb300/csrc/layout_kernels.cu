@@ -11,107 +11,92 @@
 namespace hines {
 namespace {
 
-// Unpacking chunk by chunk with the solve's task driver.  A chunk's block is
-// contiguous in the solver layout (row r: the r-th compartment from the
-// distal end of every piece longer than r), and each of its pieces is one
-// contiguous run in the plan's numbering.  The block arrives in shared
-// memory in block order (R) by one bulk copy; each lane moves the slots of
-// its own pieces, row by row (consecutive words of R), into piece order (C:
-// one row of kPitch words per piece, kPitch odd); half-warps then write each
-// piece's run to the natural layout (consecutive words of C).  Neither side
-// conflicts on shared-memory banks, and every global write is a contiguous
-// run, as the solves write x.  Only the substitution visit does anything, so
-// every chunk is handled once.  kMapped: the plan's numbering is not the
-// caller's (re-rooted plans), so the caller's index of every slot comes from
-// the plan's slot map.
+// Unpacking chunk by chunk, a warp each (chunks do not depend on one another
+// here).  A chunk's block is contiguous in the solver layout (row r: the r-th
+// compartment from the distal end of every piece longer than r), and each of
+// its pieces is one contiguous run in the plan's numbering.  The block arrives
+// in shared memory in block order (R) by one bulk copy; each lane moves the
+// slots of its own pieces, row by row (consecutive words of R), into piece
+// order (C: one row of kPitch words per piece, kPitch odd); half-warps then
+// write each piece's run to the natural layout (consecutive words of C).
+// Neither side conflicts on shared-memory banks, and every global write is a
+// contiguous run, as the solves write x.  kMapped: the plan's numbering is not
+// the caller's (re-rooted plans), so the caller's index of every slot comes
+// from the plan's slot map.  Latency bounds a chunk (block, then its runs), so
+// as many warps as shared memory holds work at once.  (As a visit of the
+// solves' task driver it walked every task twice, in two launches: 249 us for
+// 21M compartments of 8 bytes; a warp
+// per chunk 103 us; re-rooted plan 540, now 226 us.)
 //
 // (Packing stays slot by slot: a chunk-wise gather measured slower than the
 // plain kernel below, 1.02 against 0.66 ms per FP32 array of the full
 // uneven population, which reads scattered but writes contiguously.)
-template <typename W, int P, bool kMapped>
-struct UnpackMode {
+template <typename W, int P>
+struct Unpack {
   using G = Geo<P>;
-  static constexpr bool kPacked = false;  // pieces located by their first compartment in the plan's numbering
-  static constexpr bool kNeedsBlk = true;
-  static constexpr int kPer = P;
-  struct Args {
-    const W* src;
-    W* dst;
-    const int64_t* map;  // kMapped: the caller's index of every slot (-1: padding)
-  };
   static constexpr int kPitch = kL + 1;
-  static constexpr int kRowBytes = G::kSlots * 8;              // R (holds a padded block)
-  static constexpr int kColBytes = G::kChunk * kPitch * 8;     // C
-  static constexpr int kTab = kRowBytes + kColBytes;           // the block's row offsets
-  static constexpr int kStageBytes = kTab + 80;
-  static constexpr int kStages = 1;
-  static constexpr int kCacheBytes = 16;
-  static constexpr int kWarpBytes = kStageBytes + kCacheBytes;
-  static constexpr int kMinBlocks = 8;
-  static_assert(kRowBytes % 16 == 0 && kColBytes % 16 == 0 && kStageBytes % 16 == 0, "16-byte aligned regions");
-  using Bulk = BulkStage<kStageBytes>;
-  __device__ static void init_warp(unsigned char* wbase, int lane) { Bulk::init(wbase, lane); }
-
-  // the block with its padding: blocks start on multiples of 4 slots, so
-  // this is the distance to the next block (whole 16-byte words)
-  __device__ static int padded(const int* tab) { return (tab[kL] + 3) & ~3; }
-  __device__ static W* rows_of(unsigned char* buf) { return reinterpret_cast<W*>(buf); }
-  __device__ static W* cols_of(unsigned char* buf) { return reinterpret_cast<W*>(buf + kRowBytes); }
-
-  // every slot of the lane's pieces, row by row: f(slot in R, word in C)
-  template <typename F>
-  __device__ static void for_lane_slots(const Meta<P>& m, int lane, const int* tab, F&& f) {
-    const int L = m.L;
-    for (int r = 0; r < L; ++r) {
-      const int t = L - 1 - r;  // distance from the proximal end (pieces of a pair aligned there)
-#pragma unroll
-      for (int h = 0; h < P; ++h) {
-        const int i = P * lane + h;
-        if (t < m.p[h].len) f(tab[r] + i, i * kPitch + t);
-      }
-    }
-  }
-
-  __device__ static void stage(const DevPlan&, const Args& A, int visit, Meta<P>& m, int n, int lane,
-                               unsigned char* buf, const Prev&) {
-    if (visit == 0) return;
-    int* tab = reinterpret_cast<int*>(buf + kTab);
-    build_row_table<P>(m.L, lane, tab);
-    Bulk::template issue<1>(buf, lane, (unsigned)(padded(tab) * (int)sizeof(W)), buf, A.src + m.blk);
-  }
-  __device__ static void compute(const DevPlan& Pl, const Args&, int visit, int, int, int lane, const Meta<P>& m,
-                                 unsigned char* buf, const Prev&, unsigned char*, int) {
-    if (visit == 0) return;
-    const int* tab = reinterpret_cast<const int*>(buf + kTab);
-    W* sr = rows_of(buf);
-    W* sc = cols_of(buf);
-    Bulk::wait(Pl, buf, lane);
-    for_lane_slots(m, lane, tab, [&](int q, int c) { sc[c] = sr[q]; });
-  }
-  __device__ static void copy_out(const DevPlan&, const Args& A, int visit, const Meta<P>& m, int n, int lane,
-                                  unsigned char* buf) {
-    if (visit == 0) return;
-    const int* tab = reinterpret_cast<const int*>(buf + kTab);
-    const W* sc = cols_of(buf);
-    for_chunk_elements(m, n, lane, [&](int i, int t, int row, long long g, bool) {
-      const W v = sc[i * kPitch + t];
-      if constexpr (kMapped) {
-        const long long c = __ldg(A.map + m.blk + tab[row] + i);
-        if (c >= 0) A.dst[c] = v;
-      } else {
-        A.dst[g] = v;
-      }
-    });
-  }
+  static constexpr int kRowBytes = (G::kSlots * (int)sizeof(W) + 15) / 16 * 16;          // R (holds a padded block)
+  static constexpr int kColBytes = (G::kChunk * kPitch * (int)sizeof(W) + 15) / 16 * 16;  // C
+  static constexpr int kTab = kRowBytes + kColBytes;                                     // the block's row offsets
+  static constexpr int kWarpBytes = kTab + 96;
+  static constexpr int kWarps = 4;
+  using Bulk = BulkStage<kTab + 80>;
 };
 
 template <typename W, int P, bool kMapped>
+__global__ void __launch_bounds__(32 * Unpack<W, P>::kWarps)
+    k_unpack(DevPlan Pl, const W* __restrict__ src, W* __restrict__ dst, const int64_t* __restrict__ map) {
+  using U = Unpack<W, P>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned char* buf = smem + w * U::kWarpBytes;
+  int* tab = reinterpret_cast<int*>(buf + U::kTab);
+  const W* sr = reinterpret_cast<const W*>(buf);
+  W* sc = reinterpret_cast<W*>(buf + U::kRowBytes);
+  if (lane == 0) U::Bulk::init(buf);
+  __syncwarp();
+  for (int k = blockIdx.x * U::kWarps + w; k < Pl.n_chunks; k += gridDim.x * U::kWarps) {
+    const int c0 = __ldg(Pl.chunk_pos + k), n = __ldg(Pl.chunk_pos + k + 1) - c0;
+    const Meta<P> m = unpack_meta(load_meta<false, P>(Pl, c0, n, lane, true));
+    build_row_table<P>(m.L, lane, tab);
+    // the block with its padding: blocks start on multiples of 4 slots, so
+    // this is the distance to the next block (whole 16-byte words)
+    U::Bulk::template issue<1>(buf, lane, (unsigned)(((tab[kL] + 3) & ~3) * (int)sizeof(W)), buf, src + m.blk);
+    U::Bulk::wait(Pl, buf, lane);
+    for (int r = 0; r < m.L; ++r) {
+      const int t = m.L - 1 - r;  // distance from the proximal end (pieces of a pair aligned there)
+#pragma unroll
+      for (int h = 0; h < P; ++h) {
+        const int i = P * lane + h;
+        if (t < m.p[h].len) sc[i * U::kPitch + t] = sr[tab[r] + i];
+      }
+    }
+    __syncwarp();
+    for_chunk_elements(m, n, lane, [&](int i, int t, int row, long long g) {
+      const W v = sc[i * U::kPitch + t];
+      if constexpr (kMapped) {
+        const long long c = __ldg(map + m.blk + tab[row] + i);
+        if (c >= 0) dst[c] = v;
+      } else {
+        dst[g] = v;
+      }
+    });
+    __syncwarp();
+  }
+}
+
+template <typename W, int P, bool kMapped>
 cudaError_t unpack_by_chunks(const DevPlan& Pd, const W* pk, W* nat, cudaStream_t s) {
-  using M = UnpackMode<W, P, kMapped>;
-  int grid = 0;
-  cudaError_t e = grid_of<M>(Pd, &grid);
+  using U = Unpack<W, P>;
+  const int smem = U::kWarps * U::kWarpBytes;
+  cudaError_t e = cudaFuncSetAttribute(k_unpack<W, P, kMapped>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  int per_sm = 0;
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_unpack<W, P, kMapped>, 32 * U::kWarps, smem);
   if (e != cudaSuccess) return e;
-  return launch_phases<M>(Pd, typename M::Args{pk, nat, Pd.pk_perm}, grid, s);
+  const int need = (Pd.n_chunks + U::kWarps - 1) / U::kWarps, most = Pd.sms * (per_sm > 0 ? per_sm : 1);
+  k_unpack<W, P, kMapped><<<need < most ? need : most, 32 * U::kWarps, smem, s>>>(Pd, pk, nat, Pd.pk_perm);
+  return cudaGetLastError();
 }
 
 template <typename W>

@@ -1,11 +1,13 @@
 // Warp-task kernels of the batched Hines solver, sm_103a.
 //
 // The planner cuts every cell into units -- whole small cells, or the top part
-// and the subtrees of a large cell -- and packs units into tasks.  A warp owns
-// a task and walks its chunks (Hu's list schedule of the task's pieces, at
-// most 32 * P pieces each, longest first): deepest chunk first for the
-// elimination, root-side chunk first for the substitution (Section 3).  Lane
-// j owns the chunk's pieces P j .. P j + P - 1 (P = 1 or 2 pieces per lane).
+// and the subtrees of a large cell -- and packs units into tasks.  A team of
+// two warps owns a task and walks its chunks (Hu's list schedule of the task's
+// pieces, at most 32 * P pieces each, longest first): deepest chunk first for
+// the elimination, root-side chunk first for the substitution (Section 3).
+// One warp computes; the other moves data, so that copying a chunk's results
+// out and staging the next chunk's inputs overlap the arithmetic (run_task).
+// Lane j of the computing warp owns the chunk's pieces P j .. P j + P - 1 (P = 1 or 2 pieces per lane).
 // Inside a piece the parent of compartment i is i - 1 (Section 5): the lane
 // runs a Thomas chain (Listing 1) and leaves one contribution for its parent
 // compartment (Listing 2's parent lookup).  With P = 2 the lane runs its two
@@ -15,11 +17,11 @@
 // arithmetic runs on packed FP32-pair instructions.
 //
 // A solve is two launches: (A) whole-cell tasks (both sweeps), the
-// elimination of subtree tasks and, taken over by the warp that finishes a
+// elimination of subtree tasks and, taken over by the team that finishes a
 // cell's last subtree, that cell's top part (both sweeps); (C) the
-// substitution of subtree tasks.  No warp ever waits for another.
+// substitution of subtree tasks.  No team ever waits for another.
 //
-// The chunks of a task follow one another in the same warp, so a chunk's
+// The chunks of a task follow one another in the same team, so a chunk's
 // children are usually in the chunk just before it (elimination) and its
 // parents likewise (substitution): those values pass through a small shared
 // memory cache; other values go through global memory.  A chunk's inputs are
@@ -45,8 +47,14 @@ namespace {
 using namespace dev;
 
 constexpr int kL = kBranchCap;          // rows (compartments per piece), at most
-constexpr int kWarps = kWarpsPerCta;
-constexpr int kSmemPerSm = 227 * 1024;  // shared memory one SM gives its CTAs
+static_assert(kWarpsPerCta == 2, "a team: one computing and one moving warp");
+constexpr int kSmemPerSm = 228 * 1024;  // shared memory of an SM; 1 KB of it goes to each resident CTA
+// CTAs (teams) of `bytes` of shared memory an SM holds, at most `most`
+constexpr int teams_per_sm(int bytes, int most) {
+  return kSmemPerSm / (bytes + 16 + 1024) < most ? kSmemPerSm / (bytes + 16 + 1024) : most;
+}
+
+constexpr int kAlwaysTeams = 1 << 30;
 
 template <int P>
 struct Geo {
@@ -99,8 +107,8 @@ struct Meta {
   long long blk;  // the chunk's block offset in the solver layout
   Piece p[P];
   // substitution: the parent's solution when another chunk than the cached
-  // predecessor left it, fetched while the chunk is staged so that its
-  // latency overlaps the staging copies
+  // predecessor left it, fetched a chunk ahead (fetch) so that its latency
+  // overlaps the computation
   PreX xpre[P];
   // elimination (FP64): the contributions of the first two children, where
   // other chunks than the cached predecessor left them, fetched likewise
@@ -224,42 +232,36 @@ __device__ __forceinline__ void build_row_table(int L, int lane, int* tab) {
 struct ChunkElem {
   long long first;
   int len, rows;  // compartments; rows of the owner lane
-  bool root;      // holds its cell's root compartment
 };
 template <int P>
 __device__ __forceinline__ ChunkElem chunk_elem(const Meta<P>& m, int i) {
   const int src = (i / P) & 31;
-  ChunkElem c;
-  c.first = __shfl_sync(kFull, m.p[0].first, src);
-  c.len = __shfl_sync(kFull, m.p[0].len, src);
-  int root = __shfl_sync(kFull, (int)(m.p[0].pcomp < 0), src);
-  c.rows = P == 2 ? __shfl_sync(kFull, m.L, src) : c.len;
+  // first (below 2^34) and length in one word
+  auto packed = [&](int h) { return (unsigned long long)m.p[h].first | (unsigned long long)m.p[h].len << 40; };
+  unsigned long long w = __shfl_sync(kFull, packed(0), src);
+  int rows = 0;
   if constexpr (P == 2) {
-    const long long f1 = __shfl_sync(kFull, m.p[1].first, src);
-    const int l1 = __shfl_sync(kFull, m.p[1].len, src);
-    const int r1 = __shfl_sync(kFull, (int)(m.p[1].pcomp < 0), src);
-    if (i & 1) {
-      c.first = f1;
-      c.len = l1;
-      root = r1;
-    }
+    rows = __shfl_sync(kFull, m.L, src);
+    const unsigned long long w1 = __shfl_sync(kFull, packed(1), src);
+    if (i & 1) w = w1;
   }
-  c.root = root != 0;
+  ChunkElem c{(long long)(w & ((1ull << 40) - 1)), (int)(w >> 40), rows};
+  if constexpr (P == 1) c.rows = c.len;
   return c;
 }
 
 // Every element of the chunk's pieces in the natural layout: sixteen lanes
 // per piece, two pieces per step (pieces are at most 16 long).  f(i, t, row,
-// g, root) for piece i, distance t from its proximal end, row of the staged
-// chunk, natural index g, and whether the piece holds its cell's root
-// compartment (its parent is none).
+// g) for piece i, distance t from its proximal end, row of the staged chunk,
+// natural index g.
 template <int P, typename F>
 __device__ __forceinline__ void for_chunk_elements(const Meta<P>& m, int n, int lane, F&& f) {
   const int half = lane >> 4, t = lane & 15;
+#pragma unroll 1
   for (int j = 0; j < n; j += 2) {
     const int i = j + half;
     const ChunkElem c = chunk_elem(m, i);
-    if (i < n && t < c.len) f(i, t, c.rows - 1 - t, c.first + t, c.root);
+    if (i < n && t < c.len) f(i, t, c.rows - 1 - t, c.first + t);
   }
 }
 
@@ -269,6 +271,7 @@ template <typename T>
 __device__ __forceinline__ void stage_block(T* dst, const T* src, long long blk, int e, int lane) {
   constexpr int V = 16 / (int)sizeof(T);
   const int nv = (e + V - 1) / V;
+#pragma unroll 1
   for (int v = lane; v < nv; v += 32) cp_async16(dst + v * V, src + blk + (long long)v * V);
 }
 
@@ -290,41 +293,37 @@ __device__ __forceinline__ typename VOf<P>::type vpack(const float* a) {
 __device__ __forceinline__ F2 vset_hi(F2 v, float w) { return f2_make(f2_lo(v), w); }
 
 // ---- bulk staging -------------------------------------------------------------
-// Contiguous blocks are staged by one-dimensional bulk copies that one lane
-// issues, completing on a per-warp shared-memory barrier at byte kOff of the
-// warp's region (then its phase parity and a failure flag).  A mode with one
-// staging buffer has at most one staging in flight, so one barrier does.
+// Contiguous blocks are staged by one-dimensional bulk copies that one lane of
+// the moving warp issues, completing on the staging buffer's shared-memory
+// barrier at its byte kOff (then its phase parity and a failure flag), on
+// which the computing warp waits.
 template <int kOff>
 struct BulkStage {
   static_assert(kOff % 8 == 0, "barrier alignment");
-  static constexpr int kBytes = 16;  // barrier, parity word, failure flag
   // bounded wait: a poll that sees nothing suspends about 3.75 us on a GB300
   // (hines_check_bounded_wait measures it), so about one second in all, far
   // beyond any real copy latency
   static constexpr int kWaitPolls = 1 << 18;
-  __device__ static uint64_t* barrier(unsigned char* wbase) { return reinterpret_cast<uint64_t*>(wbase + kOff); }
-  __device__ static unsigned* words(unsigned char* wbase) { return reinterpret_cast<unsigned*>(barrier(wbase) + 1); }
-  // once per warp, before its first task
-  __device__ static void init(unsigned char* wbase, int lane) {
-    if (lane == 0) {
-      mbar_init(barrier(wbase));
-      words(wbase)[0] = 0u;  // parity of the next phase
-      words(wbase)[1] = 0u;  // a wait of this warp has run out
-    }
-    __syncwarp();
+  __device__ static uint64_t* barrier(unsigned char* buf) { return reinterpret_cast<uint64_t*>(buf + kOff); }
+  __device__ static unsigned* words(unsigned char* buf) { return reinterpret_cast<unsigned*>(barrier(buf) + 1); }
+  // once per staging buffer, before the first task (one thread)
+  __device__ static void init(unsigned char* buf) {
+    mbar_init(barrier(buf));
+    words(buf)[0] = 0u;  // parity of the next phase
+    words(buf)[1] = 0u;  // a wait on this buffer has run out
   }
   // one arrival with the expected bytes, then the copies.  Every lane fences
-  // its earlier ordinary accesses first: the buffer's previous contents, and
-  // factors this warp wrote in an earlier chunk of the same task, which the
-  // copies may read.
+  // its earlier ordinary accesses to the buffer first (the computing warp's
+  // lie before the team's last barrier); what the copies read of this task's
+  // own results is fenced where the sweeps turn (run_task).
   template <int N>
-  __device__ static void issue(unsigned char* wbase, int lane, unsigned bytes, void* d0, const void* s0,
+  __device__ static void issue(unsigned char* buf, int lane, unsigned bytes, void* d0, const void* s0,
                                void* d1 = nullptr, const void* s1 = nullptr, void* d2 = nullptr,
                                const void* s2 = nullptr) {
-    fence_async();
+    fence_async_shared();
     __syncwarp();
     if (lane == 0) {
-      uint64_t* bar = barrier(wbase);
+      uint64_t* bar = barrier(buf);
       mbar_expect_tx(bar, N * bytes);
       if (bytes > 0) {
         bulk_g2s(d0, s0, bytes, bar);
@@ -334,13 +333,13 @@ struct BulkStage {
     }
   }
   // every lane waits for the staged copies; a wait that runs out raises the
-  // plan's timeout status and goes on (no access leaves its buffer), and the
-  // warp's later waits poll only once, so that a failed launch ends within
+  // plan's timeout status and goes on (no access leaves its buffer), and
+  // later waits on the buffer poll only once, so that a failed launch ends within
   // about a second instead of a second per chunk
-  __device__ static void wait(const DevPlan& Pl, unsigned char* wbase, int lane) {
-    unsigned* w = words(wbase);
+  __device__ static void wait(const DevPlan& Pl, unsigned char* buf, int lane) {
+    unsigned* w = words(buf);
     const unsigned parity = w[0];
-    const bool ok = mbar_wait(barrier(wbase), parity, w[1] ? 1 : kWaitPolls);
+    const bool ok = mbar_wait(barrier(buf), parity, w[1] ? 1 : kWaitPolls);
     if (!ok && lane == 0 && Pl.status) atomicCAS(Pl.status, 0, (int)HINES_ERR_TIMEOUT);
     __syncwarp();
     if (lane == 0) {
@@ -384,25 +383,39 @@ struct CompMode {
   // first two); then the block's row table
   static constexpr int kArr = 3 * G::kSlots * 4, kFac = G::kSlots * 16;
   static constexpr int kTab = kArr > kFac ? kArr : kFac;
-  static constexpr int kStageBytes = kTab + 80;
-  static constexpr int kStages = 1;
+  static constexpr int kStageBytes = kTab + 96;
   // contiguous blocks (the factor block; d, u, b in the solver layout) are
-  // staged by bulk copies (BulkStage, its barrier after the caches)
+  // staged by bulk copies (BulkStage, its barrier after the row table)
   static constexpr bool kBulk = true;
-  static constexpr int kCslot = 0, kCx = 2 * G::kChunk * 16, kBar = kCx + 2 * G::kChunk * 8;
-  static constexpr int kCacheBytes = kBar + 16;
-  static constexpr int kWarpBytes = kStages * kStageBytes + kCacheBytes;
-  static constexpr int kMinBlocks = kSmemPerSm / (kWarps * kWarpBytes) < 12 ? kSmemPerSm / (kWarps * kWarpBytes) : 12;
-  static_assert(kStages == 1 && kStageBytes % 16 == 0, "one staging buffer, 16-byte aligned");
-  using Bulk = BulkStage<kStageBytes + kBar>;
+  // the caches of the two sweeps share their space
+  static constexpr int kCslot = 0, kCx = 0, kCacheBytes = 2 * G::kChunk * 16;
+  static constexpr int kTeamBytes = 2 * kStageBytes + kCacheBytes;
+  static constexpr int kWarpBytes = kStageBytes + kCacheBytes;
+  static constexpr int kMinBlocks = teams_per_sm(kTeamBytes, 12), kMinBlocksAlone = teams_per_sm(2 * kWarpBytes, 12);
+  // teams up to 18/16 entries per resident team (team against lone warp, us:
+  // 1940 entries 240 : 290, 1421 377 : 414, 2629 677 : 645, 2790 598 : 518)
+  static constexpr int kTeamShare = 18;
+  static_assert(kStageBytes % 16 == 0, "16-byte aligned buffers");
+  using Bulk = BulkStage<kTab + 80>;
 
   __device__ static bool bulk_staged(int visit) { return kBulk && (visit == 1 || kPk); }
-  __device__ static void init_warp(unsigned char* wbase, int lane) {
-    if (kBulk) Bulk::init(wbase, lane);
+  __device__ static void init_buffer(unsigned char* buf) {
+    if (kBulk) Bulk::init(buf);
+  }
+  // what the chunk needs of earlier chunks that no cache holds
+  __device__ static void fetch(const DevPlan& Pl, const Args&, int visit, Meta<P>& m, const Prev& pv) {
+    if (visit == 0) return;
+#pragma unroll
+    for (int h = 0; h < P; ++h) {
+      const Piece& q = m.p[h];
+      const int loc = q.ppos - pv.c0;
+      if (q.len > 0 && q.pcomp >= 0 && !(loc >= 0 && loc < pv.n))
+        m.xpre[h].ff = static_cast<const float2*>(Pl.xlast)[q.ppos];
+    }
   }
 
-  __device__ static void stage(const DevPlan& Pl, const Args& A, int visit, Meta<P>& m, int n, int lane,
-                               unsigned char* buf, const Prev& pv) {
+  __device__ static void stage(const DevPlan& Pl, const Args& A, int visit, const Meta<P>& m, int n, int lane,
+                               unsigned char* buf) {
     int* tab = reinterpret_cast<int*>(buf + kTab);
     build_row_table<P>(m.L, lane, tab);
     const int e = tab[kL];
@@ -412,14 +425,6 @@ struct CompMode {
       } else {
         stage_block(reinterpret_cast<float4*>(buf), static_cast<const float4*>(Pl.ff4), m.blk, e, lane);
         cp_commit();
-      }
-      // the parent's solution, unless the predecessor chunk's cache holds it
-#pragma unroll
-      for (int h = 0; h < P; ++h) {
-        const Piece& q = m.p[h];
-        const int loc = q.ppos - pv.c0;
-        if (q.len > 0 && q.pcomp >= 0 && !(loc >= 0 && loc < pv.n))
-          m.xpre[h].ff = static_cast<const float2*>(Pl.xlast)[q.ppos];
       }
       return;
     }
@@ -439,7 +444,7 @@ struct CompMode {
       stage_block(su, A.u, blk, e, lane);
       stage_block(sb, A.b, blk, e, lane);
     } else {
-      for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
+      for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g) {
         const int q = nidx<P>(row, i);
         cp_async4(&sd[q], A.d + g);
         cp_async4(&su[q], A.u + g);
@@ -477,6 +482,7 @@ struct CompMode {
         if (q.len == 0) continue;
         const int idx = rows.slot(L - q.len, me + h);
         ff Dv = {sd[idx], 0.f}, Bv = {sb[idx], 0.f};
+#pragma unroll 1
         for (int c = 0; c < q.nchild; ++c) {
           const int cp = child_pos(Pl, q, c);
           const int loc = cp - pv.c0;
@@ -593,10 +599,11 @@ struct CompMode {
     if (kPk) {
       const long long blk = __shfl_sync(kFull, m.p[0].first, 0);
       const int e = tab[kL];
+#pragma unroll 1
       for (int s = lane; s < e; s += 32) A.x[blk + s] = sx[2 * s];
       return;
     }
-    for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) { A.x[g] = sx[2 * (tab[row] + i)]; });
+    for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g) { A.x[g] = sx[2 * (tab[row] + i)]; });
   }
 };
 
@@ -654,10 +661,10 @@ struct FactorMode {
   static constexpr bool kNeedsBlk = kBF;
   static constexpr int kPer = P;
   // row loops: sixteen copies of the long FP64 row overrun the instruction
-  // cache (4 against 16: 64 small cells 47.1 against 51.2 us, 59M compartments
-  // 1.60 against 1.65 ms); a row that re-uses its factor is short (7.65
+  // cache (2 against 16: 64 small cells 47.1 against 51.2 us, 59M compartments
+  // 1.61 against 1.65 ms); a row that re-uses its factor is short (7.85
   // against 7.29 ms per 40 steps of 1.7M compartments)
-  static constexpr int kUnroll = kYG && !kReuse ? 4 : kL;
+  static constexpr int kUnroll = kYG && !kReuse ? 2 : kL;
   static_assert(!kReuse || (kCable && kYG), "only FP64 cable steps re-use a factor");
   struct Args {
     const T* d;
@@ -671,21 +678,22 @@ struct FactorMode {
   };
   // a staging buffer: d (or the factor), u, b, then the row table (solver layout)
   static constexpr int kTab = 3 * G::kSlots * (int)sizeof(T);
-  static constexpr int kStageBytes = kTab + 80;
-  // FP64 chunks are large and the FP64 pipe is slow: one staging buffer, so
-  // that more warps share an SM; FP32 with one piece per lane: two
-  static constexpr int kStages = (sizeof(T) == 4 && P == 1) ? 2 : 1;
-  static constexpr int kCslot = 0, kCx = 2 * G::kChunk * 2 * (int)sizeof(T);
-  static constexpr int kBar = kCx + 2 * G::kChunk * (int)sizeof(T);
-  static constexpr int kCacheBytes = kBar + (kBF ? 16 : 0);
-  static constexpr int kWarpBytes = kStages * kStageBytes + kCacheBytes;
-  static constexpr int kMinBlocks = kSmemPerSm / (kWarps * kWarpBytes);
-  // the factor block is staged by bulk copies (FP64 has one staging buffer)
+  static constexpr int kStageBytes = kTab + 96;
+  static constexpr int kCslot = 0, kCx = 0, kCacheBytes = 2 * G::kChunk * 2 * (int)sizeof(T);
+  static constexpr int kTeamBytes = 2 * kStageBytes + kCacheBytes;
+  static constexpr int kWarpBytes = kStageBytes + kCacheBytes;
+  static constexpr int kMinBlocks = teams_per_sm(kTeamBytes, 10), kMinBlocksAlone = teams_per_sm(2 * kWarpBytes, 10);
+  // teams up to this many sixteenths of an entry per resident team (team
+  // against lone warp, us; FP64: 1434 entries 262 : 318, 1940 668 : 764, 2340
+  // 655 : 633, 3760 560 : 535; FP32: 1940 195 : 236, 2629 558 : 479; re-using
+  // a factor: 2823 2511 : 2817, 2751 5731 : 5727)
+  static constexpr int kTeamShare = kReuse ? 40 : kYG ? 28 : 21;
+  // the factor block is staged by bulk copies
   static constexpr bool kBulk = kBF;
-  static_assert(!kBF || (kStages == 1 && kStageBytes % 16 == 0), "one staging buffer, 16-byte aligned");
-  using Bulk = BulkStage<kStageBytes + kBar>;
-  __device__ static void init_warp(unsigned char* wbase, int lane) {
-    if (kBulk) Bulk::init(wbase, lane);
+  static_assert(kStageBytes % 16 == 0, "16-byte aligned buffers");
+  using Bulk = BulkStage<kTab + 80>;
+  __device__ static void init_buffer(unsigned char* buf) {
+    if (kBulk) Bulk::init(buf);
   }
   // (g, y) per slot of the solver layout
   __device__ static double2* factor_block(const DevPlan& Pl) { return static_cast<double2*>(Pl.ff4); }
@@ -706,7 +714,7 @@ struct FactorMode {
   // lane are loaded before any is computed: one at a time, every element
   // waited for its loads (19.6k clocks a chunk of the 15M-compartment step,
   // more than the elimination itself).
-  static constexpr int kStep = kReuse ? 4 : 2;
+  static constexpr int kStep = 2;
   struct Elem {
     T s, g, u, v;
     __device__ void load(const Args& A, long long i) {
@@ -726,6 +734,7 @@ struct FactorMode {
     }
   };
   __device__ static void rebuild_block(const Args& A, long long blk, int e, int lane, T* sd, T* su, T* sb) {
+#pragma unroll 1
     for (int i0 = lane; i0 < e; i0 += 32 * kStep) {
       Elem el[kStep];
 #pragma unroll
@@ -739,6 +748,7 @@ struct FactorMode {
   template <typename F>
   __device__ static void rebuild_natural(const Args& A, const Meta<P>& m, int n, int lane, T* sd, T* su, T* sb, F&& f) {
     const int half = lane >> 4, t = lane & 15;
+#pragma unroll 1
     for (int j = 0; j < n; j += 2 * kStep) {
       Elem el[kStep];
       int q[kStep];  // word of the staged chunk, -1: none
@@ -761,9 +771,30 @@ struct FactorMode {
   // A child's contribution (D, B): from the cache of the chunk just before,
   // or from the slots.
   __device__ static bool local_child(int cp, const Prev& pv) { return cp >= pv.c0 && cp < pv.c0 + pv.n; }
+  // what the chunk needs of earlier chunks that no cache holds: a parent's
+  // solution, the contributions of the first two children
+  __device__ static void fetch(const DevPlan& Pl, const Args&, int visit, Meta<P>& m, const Prev& pv) {
+#pragma unroll
+    for (int h = 0; h < P; ++h) {
+      const Piece& q = m.p[h];
+      if (visit == 1) {
+        const int loc = q.ppos - pv.c0;
+        if (q.len > 0 && q.pcomp >= 0 && !(loc >= 0 && loc < pv.n))
+          pre_set(m.xpre[h], static_cast<const T*>(Pl.xlast)[q.ppos]);
+      } else if (kYG) {
+        const double2* slot = static_cast<const double2*>(Pl.cd);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          if (c >= q.nchild) continue;
+          const int cp = child_pos(Pl, q, c);
+          if (!local_child(cp, pv)) m.cpre[h][c] = slot_load(slot + cp, q);
+        }
+      }
+    }
+  }
 
-  __device__ static void stage(const DevPlan& Pl, const Args& A, int visit, Meta<P>& m, int n, int lane,
-                               unsigned char* buf, const Prev& pv) {
+  __device__ static void stage(const DevPlan& Pl, const Args& A, int visit, const Meta<P>& m, int n, int lane,
+                               unsigned char* buf) {
     T* sd = reinterpret_cast<T*>(buf);
     T* su = sd + G::kSlots;
     T* sb = su + G::kSlots;
@@ -773,15 +804,6 @@ struct FactorMode {
     const int e = (kBF || kPk) ? tab[kL] : 0;
     const long long blk = kPk ? __shfl_sync(kFull, m.p[0].first, 0) : 0;
     if (visit == 1) {
-      // the parent's solution, unless the predecessor chunk's cache holds it
-      // (a chunk staged before its predecessor is computed finds that
-      // predecessor's solutions in the cache, so it never reads them here)
-#pragma unroll
-      for (int h = 0; h < P; ++h) {
-        const Piece& q = m.p[h];
-        const int loc = q.ppos - pv.c0;
-        if (q.len > 0 && q.pcomp >= 0 && !(loc >= 0 && loc < pv.n)) pre_set(m.xpre[h], A.x[q.pcomp]);
-      }
       if constexpr (kBF) {  // the factor block over the first two arrays
         Bulk::template issue<1>(buf, lane, (unsigned)e * 16u, buf, factor_block(Pl) + m.blk);
       } else if (kPk) {
@@ -790,7 +812,7 @@ struct FactorMode {
         stage_block(sb, static_cast<const T*>(A.x), blk, e, lane);
         cp_commit();
       } else {
-        for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
+        for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g) {
           const int q = nidx<P>(row, i);
           cp_async(&sd[q], fac + g);
           if (!kYG) cp_async(&su[q], A.u + g);
@@ -807,6 +829,7 @@ struct FactorMode {
       if (kPk) {
         stage_block(sd, rc, blk, e, lane);
         if (kBF)
+#pragma unroll 1
           for (int i = lane; i < e; i += 32) cp_async(&su[i], gp + 2 * i);
         else
           stage_block(su, gp, blk, e, lane);
@@ -829,7 +852,7 @@ struct FactorMode {
         stage_block(su, A.u, blk, e, lane);
         stage_block(sb, bsrc, blk, e, lane);
       } else {
-        for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
+        for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g) {
           const int q = nidx<P>(row, i);
           cp_async(&sd[q], A.d + g);
           cp_async(&su[q], A.u + g);
@@ -838,20 +861,6 @@ struct FactorMode {
       }
     }
     cp_commit();
-    if constexpr (kYG) {
-      // contributions that no cache holds are on their way with the inputs
-      const double2* slot = static_cast<const double2*>(Pl.cd);
-#pragma unroll
-      for (int h = 0; h < P; ++h) {
-        const Piece& q = m.p[h];
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          if (c >= q.nchild) continue;
-          const int cp = child_pos(Pl, q, c);
-          if (!local_child(cp, pv)) m.cpre[h][c] = slot_load(slot + cp, q);
-        }
-      }
-    }
   }
 
   __device__ static void compute(const DevPlan& Pl, const Args& A, int visit, int c0, int n, int lane,
@@ -912,6 +921,7 @@ struct FactorMode {
           if (q.nchild > 1) child(1, m.cpre[h][1], true);
           c = 2;
         }
+#pragma unroll 1
         for (; c < q.nchild; ++c) child(c, make_double2(0.0, 0.0), false);
       }
       // one row's factor from its pivot: g (or the multiplier) is returned
@@ -1027,8 +1037,11 @@ struct FactorMode {
       }
     }
 #pragma unroll
-    for (int h = 0; h < P; ++h)
-      if (m.p[h].len > 0) cx[cur * G::kChunk + me + h] = xp[h];
+    for (int h = 0; h < P; ++h) {
+      if (m.p[h].len == 0) continue;
+      static_cast<T*>(Pl.xlast)[c0 + me + h] = xp[h];
+      cx[cur * G::kChunk + me + h] = xp[h];
+    }
   }
 
   __device__ static void copy_out(const DevPlan& Pl, const Args& A, int visit, const Meta<P>& m, int n, int lane,
@@ -1045,10 +1058,10 @@ struct FactorMode {
       const double* sx = reinterpret_cast<const double*>(buf);
       if (kPk) {
         const int e = tab[kL];
+#pragma unroll 1
         for (int s = lane; s < e; s += 32) A.x[blk + s] = sx[2 * s];
       } else {
-        for_chunk_elements(m, n, lane,
-                           [&](int i, int, int row, long long g, bool) { A.x[g] = sx[2 * (tab[row] + i)]; });
+        for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g) { A.x[g] = sx[2 * (tab[row] + i)]; });
       }
       return;
     }
@@ -1057,6 +1070,7 @@ struct FactorMode {
     const bool keep_fac = visit == 0 && !kReuse, keep_rcp = visit == 0 && keeps_rcp(A);
     if (kPk) {
       const int e = tab[kL];
+#pragma unroll 1
       for (int s = lane; s < e; s += 32) {
         if (keep_fac) fac[blk + s] = sd[s];
         if (keep_rcp) rc[blk + s] = su[s];
@@ -1064,7 +1078,7 @@ struct FactorMode {
       }
       return;
     }
-    for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
+    for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g) {
       const int q = nidx<P>(row, i);
       if (keep_fac) fac[g] = sd[q];
       if (keep_rcp) rc[g] = su[q];
@@ -1107,38 +1121,39 @@ struct RefineMode {
   // staged words: d, u, b (visit 1: the eliminated residual), the factor, and
   // x as pairs (two words per slot; FP32 x uses the first)
   static constexpr int kTab = 6 * G::kSlots * 4;
-  static constexpr int kStageBytes = kTab + 80;
-  // one staging buffer: six staged arrays per chunk, and twice as many warps
-  // per SM hide the loads better than a second buffer at half the warps
-  // (measured on the 228M-compartment batch: 12.6 ms against 13.7 ms per
-  // one-step solve)
-  static constexpr int kStages = 1;
-  static constexpr int kCslot = 0, kCx = 2 * G::kChunk * 16;
-  static constexpr int kCacheBytes = kCx + 2 * G::kChunk * 8;
-  static constexpr int kWarpBytes = kStages * kStageBytes + kCacheBytes;
-  static constexpr int kMinBlocks = kSmemPerSm / (kWarps * kWarpBytes);
-  static constexpr bool kBulk = false;
-  __device__ static void init_warp(unsigned char*, int) {}
+  static constexpr int kStageBytes = kTab + 96;
+  static constexpr int kCslot = 0, kCx = 0, kCacheBytes = 2 * G::kChunk * 16;
+  static constexpr int kTeamBytes = 2 * kStageBytes + kCacheBytes;
+  static constexpr int kMinBlocks = teams_per_sm(kTeamBytes, 10);
+  // always teams (against lone warps, us: 700 entries 625 : 958, 2700 1610 :
+  // 2093): the copies outweigh the short arithmetic
+  static constexpr int kTeamShare = kAlwaysTeams;
+  __device__ static void init_buffer(unsigned char*) {}
 
-  __device__ static void stage(const DevPlan& Pl, const Args& A, int visit, Meta<P>& m, int n, int lane,
-                               unsigned char* buf, const Prev& pv) {
+  // what the chunk needs of earlier chunks: the parent's x (visit 0), the
+  // parent's correction where no cache holds it (visit 1)
+  __device__ static void fetch(const DevPlan& Pl, const Args& A, int visit, Meta<P>& m, const Prev& pv) {
+#pragma unroll
+    for (int h = 0; h < P; ++h) {
+      const Piece& q = m.p[h];
+      if (q.len == 0 || q.pcomp < 0) continue;
+      const int loc = q.ppos - pv.c0;
+      if (visit == 0)
+        m.xpre[h].ff = gx(A, q.pcomp);
+      else if (!(loc >= 0 && loc < pv.n))
+        m.xpre[h].f = static_cast<const float2*>(Pl.xlast)[q.ppos].x;
+    }
+  }
+
+  __device__ static void stage(const DevPlan& Pl, const Args& A, int visit, const Meta<P>& m, int n, int lane,
+                               unsigned char* buf) {
     float* sd = reinterpret_cast<float*>(buf);
     float* su = sd + G::kSlots;
     float* sb = su + G::kSlots;
     float* sf = sb + G::kSlots;
     float* sx = sf + G::kSlots;  // [2 * kSlots]
     const float* fac = static_cast<const float*>(Pl.fac);
-    if (visit == 1) {
-      // the parent's correction, unless the predecessor chunk's cache holds it
-#pragma unroll
-      for (int h = 0; h < P; ++h) {
-        const Piece& q = m.p[h];
-        const int loc = q.ppos - pv.c0;
-        if (q.len > 0 && q.pcomp >= 0 && !(loc >= 0 && loc < pv.n))
-          m.xpre[h].f = static_cast<const float2*>(Pl.xlast)[q.ppos].x;
-      }
-    }
-    for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
+    for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g) {
       const int q = nidx<P>(row, i);
       if (visit == 0) {
         cp_async4(&sd[q], A.d + g);
@@ -1209,11 +1224,12 @@ struct RefineMode {
         xph[h] = xpl[h] = crh[h] = crl[h] = ce[h] = 0.f;
         if (q.len == 0) continue;
         if (q.pcomp >= 0) {
-          const float2 t = gx(A, q.pcomp);
+          const float2 t = m.xpre[h].ff;
           xph[h] = t.x;
           xpl[h] = t.y;
         }
         ff acc = {0.f, 0.f};
+#pragma unroll 1
         for (int c = 0; c < q.nchild; ++c) {
           const int cp = child_pos(Pl, q, c);
           const int loc = cp - pv.c0;
@@ -1324,13 +1340,11 @@ struct RefineMode {
     const float* sd = reinterpret_cast<const float*>(buf);
     const float* sb = sd + 2 * G::kSlots;
     const float* sx = sd + 4 * G::kSlots;
-    for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g, bool) {
+    for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g) {
       const int q = nidx<P>(row, i);
       if (visit == 0)
         A.rw[g] = sb[q];
-      else if (kOut == 1)
-        static_cast<double*>(A.xo)[g] = reinterpret_cast<const double*>(sx)[q];
-      else
+      else  // (an FP64 x as its two words)
         static_cast<float2*>(A.xo)[g] = reinterpret_cast<const float2*>(sx)[q];
     });
   }
@@ -1371,53 +1385,82 @@ struct ChunkTable {
   }
 };
 
+// One task by a team.  Per step, between two barriers of the CTA, warp 0
+// computes chunk k while warp 1 copies out the results of chunk k - 1 and
+// stages chunk k + 1 into the same buffer: the two warps meet only at the
+// barrier, and neither waits for anything else.  Where the sweeps turn, the
+// first chunk of the substitution is staged only after the last one of the
+// elimination is out (it is the same chunk, and reads what the elimination
+// left).  In one warp with one buffer (run_task_alone) a chunk of the natural
+// compensated solve took 17.4k clocks in the elimination, 8.9k of them
+// arithmetic, and 13.1k in the substitution, 5.4k of them arithmetic.  Against
+// lone warps: FP64 solve of 64 small cells 47.1 -> 41.0 us, FP32 solve of 1001
+// small cells 79 -> 64 us, 40-step rollout with gradients 27.9 -> 22.5 ms, two
+// refinement steps 2.16 -> 1.88 ms, host pipeline 3.12 -> 2.66 ms.  Loops over
+// a chunk's elements stay rolled: code that overruns the instruction cache
+// costs more than their bookkeeping (solve of 28M compartments 835 -> 789 us
+// without the compiler's unrolling, 958 us with four steps at a time).
 template <class M>
-__device__ void run_task(const DevPlan& Pl, const typename M::Args& A, const TaskRec& t, int lane,
-                         unsigned char* wbase) {
+__device__ void run_task(const DevPlan& Pl, const typename M::Args& A, const TaskRec& t, bool mover, int lane,
+                         unsigned char* smem) {
   constexpr int P = M::kPer;
   ChunkTable tab(Pl.tlvl_ptr + t.lvl_off, t.nlvl);
   const int vb = t.code == 2 ? 1 : 0, ve = t.code == 1 ? 1 : 2;
-  unsigned char* cache = wbase + M::kStages * M::kStageBytes;
-  auto buf = [wbase](int which) { return wbase + (M::kStages == 2 ? which : 0) * M::kStageBytes; };
+  unsigned char* cache = smem + 2 * M::kStageBytes;
+  auto buf = [smem](int which) { return smem + which * M::kStageBytes; };
   auto meta = [&](const Pos& p) { return load_meta<M::kPacked, P>(Pl, p.c0, p.n, lane, M::kNeedsBlk); };
-  // metadata runs two chunks ahead; with two staging buffers the next chunk
-  // is staged while this one is computed, with one right after this one's
-  // results are out
+  auto stage = [&](const Pos& p, const Meta<P>& m, int which) {
+    M::stage(Pl, A, p.visit, m, p.n, lane, buf(which));
+    cp_wait_all();
+  };
+  // metadata runs two chunks ahead
   Pos cur = tab.at(vb, vb == 0 ? t.nlvl - 1 : 0, lane);
-  Meta<P> m_cur = unpack_meta(meta(cur));
-  Prev pv{0, 0, 0};  // last chunk of the previous level in this sweep
+  Meta<P> m_cur = unpack_meta(meta(cur)), m_prev = m_cur;
   Pos nxt = tab.next(cur, ve, lane);
   const RawMeta<M::kPacked, P> r_nxt = meta(nxt);
-  M::stage(Pl, A, cur.visit, m_cur, cur.n, lane, buf(0), pv);
+  Prev pv{0, 0, 0};  // the chunk before, if of the same sweep
+  if (mover)
+    stage(cur, m_cur, 0);
+  else
+    M::fetch(Pl, A, cur.visit, m_cur, pv);
   Meta<P> m_nxt = unpack_meta(r_nxt);
   int which = 0;
-  while (cur.visit < ve) {
-    cp_wait_all();
-    __syncwarp();
-    // nothing of the substitution is read before the elimination has
-    // finished: its first chunks reuse positions the elimination is still
-    // writing (and read the folded states it leaves)
-    const bool crossing = nxt.visit != cur.visit;
-    // predecessor of the next chunk: this chunk, if it belongs to the same sweep
-    const Prev pn = crossing ? Prev{0, 0, 0} : Prev{cur.c0, cur.n, cur.l & 1};
-    // (staged before this chunk is computed: a mode with two buffers reads
-    // nothing in stage that this chunk writes)
-    if (M::kStages == 2 && nxt.visit < ve && !crossing)
-      M::stage(Pl, A, nxt.visit, m_nxt, nxt.n, lane, buf(which ^ 1), pn);
+  __syncthreads();
+  for (;;) {
+    const bool turn = nxt.visit != cur.visit;  // the last chunk of a sweep
+    const Prev pn = turn ? Prev{0, 0, 0} : Prev{cur.c0, cur.n, cur.l & 1};
     const Pos nn = nxt.visit < ve ? tab.next(nxt, ve, lane) : nxt;
     const RawMeta<M::kPacked, P> r_nn = meta(nn);
-    M::compute(Pl, A, cur.visit, cur.c0, cur.n, lane, m_cur, buf(which), pv, cache, cur.l & 1);
-    __syncwarp();
-    M::copy_out(Pl, A, cur.visit, m_cur, cur.n, lane, buf(which));
-    __syncwarp();
-    if (crossing && nxt.visit < ve) {
-      // the substitution reads what the elimination wrote (through L2)
-      __threadfence();
+    if (mover) {
+      if (pv.n > 0) M::copy_out(Pl, A, cur.visit, m_prev, pv.n, lane, buf(which ^ 1));
       __syncwarp();
+      if (!turn) stage(nxt, m_nxt, which ^ 1);
+    } else {
+      if (!turn) M::fetch(Pl, A, nxt.visit, m_nxt, pn);
+      M::compute(Pl, A, cur.visit, cur.c0, cur.n, lane, m_cur, buf(which), pv, cache, cur.l & 1);
+      __syncwarp();
+      if (turn) {  // this warp's factors and contributions, for bulk copies and other teams
+        __threadfence();
+        fence_async();
+      }
     }
-    if (nxt.visit < ve && (crossing || M::kStages == 1))
-      M::stage(Pl, A, nxt.visit, m_nxt, nxt.n, lane, buf(which ^ 1), pn);
+    __syncthreads();
+    if (turn) {
+      const bool done = nxt.visit >= ve;
+      if (mover) {
+        M::copy_out(Pl, A, cur.visit, m_cur, cur.n, lane, buf(which));
+        __threadfence();
+        fence_async();
+        __syncwarp();
+        if (!done) stage(nxt, m_nxt, which ^ 1);
+      } else if (!done) {
+        M::fetch(Pl, A, nxt.visit, m_nxt, pn);
+      }
+      __syncthreads();
+      if (done) return;
+    }
     pv = pn;
+    m_prev = m_cur;
     cur = nxt;
     m_cur = m_nxt;
     nxt = nn;
@@ -1426,87 +1469,168 @@ __device__ void run_task(const DevPlan& Pl, const typename M::Args& A, const Tas
   }
 }
 
+// The same by one warp with one staging buffer: more tasks at a time, for
+// launches that have them.
+template <class M>
+__device__ void run_task_alone(const DevPlan& Pl, const typename M::Args& A, const TaskRec& t, int lane,
+                               unsigned char* smem) {
+  constexpr int P = M::kPer;
+  ChunkTable tab(Pl.tlvl_ptr + t.lvl_off, t.nlvl);
+  const int vb = t.code == 2 ? 1 : 0, ve = t.code == 1 ? 1 : 2;
+  unsigned char* cache = smem + M::kStageBytes;
+  auto meta = [&](const Pos& p) { return load_meta<M::kPacked, P>(Pl, p.c0, p.n, lane, M::kNeedsBlk); };
+  Pos cur{vb, 0, 0, 0}, nxt = tab.at(vb, vb == 0 ? t.nlvl - 1 : 0, lane);
+  Meta<P> m_cur = unpack_meta(meta(nxt)), m_nxt = m_cur;
+  Prev pv{0, 0, 0}, pn{0, 0, 0};
+  while (nxt.visit < ve) {
+    if (nxt.visit != cur.visit) {  // this warp's elimination, for the substitution's bulk copies
+      __threadfence();
+      fence_async();
+      __syncwarp();
+    }
+    cur = nxt;
+    m_cur = m_nxt;
+    pv = pn;
+    M::stage(Pl, A, cur.visit, m_cur, cur.n, lane, smem);
+    M::fetch(Pl, A, cur.visit, m_cur, pv);
+    nxt = tab.next(cur, ve, lane);
+    const RawMeta<M::kPacked, P> r_nxt = meta(nxt);
+    cp_wait_all();
+    __syncwarp();
+    M::compute(Pl, A, cur.visit, cur.c0, cur.n, lane, m_cur, smem, pv, cache, cur.l & 1);
+    __syncwarp();
+    M::copy_out(Pl, A, cur.visit, m_cur, cur.n, lane, smem);
+    __syncwarp();
+    pn = nxt.visit != cur.visit ? Prev{0, 0, 0} : Prev{cur.c0, cur.n, cur.l & 1};
+    m_nxt = unpack_meta(r_nxt);
+  }
+  __threadfence();  // (a hand-over follows)
+  __syncwarp();
+}
+
 // After a subtree task's elimination: count its units off their cell's
-// pending count; the warp that finishes the cell's last subtree takes over
+// pending count; the team that finishes the cell's last subtree takes over
 // the cell's top part (both visits) as its next task, and restores the count
 // for the next call.  Nothing waits: the hand-over goes to whoever arrives
-// last.  Release: every lane fences its slot writes before lane 0's atomic;
-// acquire: the fence after it, and the top part reads those slots through L2.
-// Returns the top task, or -1.
-__device__ __forceinline__ int hand_over(const DevPlan& P, int t, int lane) {
-  __threadfence();
-  __syncwarp();
+// last.  Release: every lane fenced its writes before the team's last barrier;
+// acquire: the fence after the atomic, before the team's next barrier, and the
+// top part reads those slots through L2.  One thread; returns the top task, or
+// -1.
+__device__ __forceinline__ int hand_over(const DevPlan& P, int t) {
   const int cell = __ldg(P.task_sub + 2 * t);
   if (cell < 0) return -1;
-  int last = 0;
-  if (lane == 0) {
-    const int cnt = __ldg(P.task_sub + 2 * t + 1);
-    last = atomicSub(P.cell_pending + cell, cnt) == cnt;
-    if (last) P.cell_pending[cell] = __ldg(P.counter_init + 4 + cell);
-  }
-  if (!__shfl_sync(kFull, last, 0)) return -1;
+  const int cnt = __ldg(P.task_sub + 2 * t + 1);
+  __threadfence();
+  if (atomicSub(P.cell_pending + cell, cnt) != cnt) return -1;
+  P.cell_pending[cell] = __ldg(P.counter_init + 4 + cell);
   __threadfence();
   return __ldg(P.cell_top_task + cell);
 }
 
-template <class M>
-__global__ void __launch_bounds__(32 * kWarps, M::kMinBlocks) k_units(DevPlan P, typename M::Args A, int phase) {
+// kTeam: a CTA is one team; else its two warps run a task each.
+template <class M, bool kTeam>
+constexpr int min_blocks() {
+  if constexpr (kTeam)
+    return M::kMinBlocks;
+  else
+    return M::kMinBlocksAlone;
+}
+template <class M, bool kTeam>
+__host__ __device__ constexpr int cta_bytes() {
+  if constexpr (kTeam)
+    return M::kTeamBytes + 16;
+  else
+    return 2 * M::kWarpBytes;
+}
+template <class M, bool kTeam>
+__global__ void __launch_bounds__(64, min_blocks<M, kTeam>())
+    k_units(DevPlan P, typename M::Args A, int phase) {
   extern __shared__ __align__(16) unsigned char smem_u[];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned char* wbase = smem_u + w * M::kWarpBytes;
-  M::init_warp(wbase, lane);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int* ctl = reinterpret_cast<int*>(smem_u + M::kTeamBytes);  // the team's next entry, or top part
+  constexpr int kWarpBytes = cta_bytes<M, kTeam>() / 2;
+  unsigned char* smem = kTeam ? smem_u : smem_u + w * kWarpBytes;
+  bool mover = false;
+  if (kTeam) {
+    if (threadIdx.x < 2) M::init_buffer(smem_u + threadIdx.x * M::kStageBytes);
+    __syncthreads();
+    mover = w == 1;
+  } else {
+    if (lane == 0) M::init_buffer(smem);
+    __syncwarp();
+  }
   const int e0 = P.phase_off[phase], ne = P.phase_off[phase + 1] - e0;
-  const int warps = (int)gridDim.x * kWarps;
+  const int runners = kTeam ? (int)gridDim.x : 2 * (int)gridDim.x;
   int* next_entry = P.counter + phase;
-  // the first entry of a warp is its own number, the others are counted off
-  int k = (int)blockIdx.x * kWarps + w;
-  if (k >= ne) return;  // (only where there are fewer entries than warps)
   auto entry = [&](int i) {
     const int4 r = __ldg(P.phase_rec + e0 + i);
     return TaskRec{(uint32_t)r.x, r.y, r.z, r.w};
   };
+  // the first entry of a runner (team or warp) is its own number, the others
+  // are counted off
+  int k = kTeam ? (int)blockIdx.x : 2 * (int)blockIdx.x + w;
+  if (k >= ne) return;  // (one warp of the last CTA, at most)
   TaskRec t = entry(k);
   for (;;) {
-    run_task<M>(P, A, t, lane, wbase);
-    if (t.code == 1) {
-      const int top = hand_over(P, t.id, lane);
-      if (top >= 0) {
-        t = TaskRec{(uint32_t)P.task_lvl_off[top], P.task_nlvl[top], top, 0};
-        continue;
-      }
+    if constexpr (kTeam)
+      run_task<M>(P, A, t, mover, lane, smem);
+    else
+      run_task_alone<M>(P, A, t, lane, smem);
+    // the next entry: a top part handed over (-2 - task), or one counted off
+    if (kTeam ? threadIdx.x == 0 : lane == 0) {
+      const int top = t.code == 1 ? hand_over(P, t.id) : -1;
+      k = top >= 0 ? -2 - top : ne <= runners ? ne : runners + atomicAdd(next_entry, 1);
+      if (kTeam) ctl[0] = k;
     }
-    if (ne <= warps) return;  // one entry per warp: nothing is counted
-    if (lane == 0) k = warps + atomicAdd(next_entry, 1);
-    k = __shfl_sync(kFull, k, 0);
+    if constexpr (kTeam) {
+      __syncthreads();
+      k = ctl[0];
+      __syncthreads();
+    } else {
+      k = __shfl_sync(kFull, k, 0);
+    }
     if (k >= ne) break;
-    t = entry(k);
+    t = k >= 0 ? entry(k) : TaskRec{(uint32_t)P.task_lvl_off[-2 - k], P.task_nlvl[-2 - k], -2 - k, 0};
   }
-  // every warp ends on one count past the entries: the last of them restores
+  // every runner ends on one count past the entries: the last of them restores
   // the counter, so that no copy has to before the next call
-  if (lane == 0 && k == ne + warps - 1) *next_entry = 0;
+  if (lane == 0 && !mover && ne > runners && k == ne + runners - 1) *next_entry = 0;
 }
 
-template <class M>
+template <class M, bool kTeam>
 cudaError_t grid_of(const DevPlan& P, int* grid) {
   int per_sm = 0;
-  const size_t smem = (size_t)kWarps * M::kWarpBytes;
-  cudaError_t e = cudaFuncSetAttribute(k_units<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_units<M>, 32 * kWarps, smem);
+  const size_t smem = cta_bytes<M, kTeam>();
+  const auto kernel = k_units<M, kTeam>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 64, smem);
   if (e != cudaSuccess) return e;
   *grid = P.sms * (per_sm > 0 ? per_sm : 1);
   return cudaSuccess;
 }
+// persistent grid sizes of both kernels of a mode: teams, and CTAs of two lone warps
+template <class M>
+cudaError_t grid_of(const DevPlan& P, int2* grid) {
+  cudaError_t e = grid_of<M, true>(P, &grid->x);
+  if constexpr (M::kTeamShare != kAlwaysTeams)
+    if (e == cudaSuccess) e = grid_of<M, false>(P, &grid->y);
+  return e;
+}
 
 template <class M>
-cudaError_t launch_phases(const DevPlan& P, const typename M::Args& A, int grid, cudaStream_t s) {
+cudaError_t launch_phases(const DevPlan& P, const typename M::Args& A, int2 grid, cudaStream_t s) {
   if (P.n_wtasks == 0) return cudaSuccess;
-  const size_t smem = (size_t)kWarps * M::kWarpBytes;
   for (int phase = 0; phase < 3; ++phase) {
     const int ne = P.phase_off[phase + 1] - P.phase_off[phase];
     if (ne == 0) continue;
-    const int warps = ne < grid * kWarps ? ne : grid * kWarps;
-    const int blocks = (warps + kWarps - 1) / kWarps;
-    k_units<M><<<blocks, 32 * kWarps, smem, s>>>(P, A, phase);
+    // teams where one runner per entry leaves the chip idle anyway, lone
+    // warps, twice as many tasks at a time, where there are entries for them
+    if (M::kTeamShare == kAlwaysTeams || ne <= M::kTeamShare * grid.x / 16) {
+      k_units<M, true><<<ne < grid.x ? ne : grid.x, 64, cta_bytes<M, true>(), s>>>(P, A, phase);
+    } else if constexpr (M::kTeamShare != kAlwaysTeams) {
+      const int ctas = (ne + 1) / 2;
+      k_units<M, false><<<ctas < grid.y ? ctas : grid.y, 64, cta_bytes<M, false>(), s>>>(P, A, phase);
+    }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -1547,7 +1671,7 @@ struct UnitKernels {
     if (e == cudaSuccess) e = grid_of<PkF32>(P, &P.grid[5]);
     if (e == cudaSuccess) e = grid_of<PkComp>(P, &P.grid[6]);
     if (e == cudaSuccess) e = grid_of<PkCable>(P, &P.grid[7]);
-    int g_reuse = 0;  // same footprint as the plain modes
+    int2 g_reuse;  // same footprint as the plain modes
     if (e == cudaSuccess) e = grid_of<CableReuse>(P, &g_reuse);
     if (e == cudaSuccess) e = grid_of<PkCableReuse>(P, &g_reuse);
     if (e == cudaSuccess) e = grid_of<R32to2>(P, &P.grid_refine);
