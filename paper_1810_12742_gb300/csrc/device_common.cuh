@@ -103,30 +103,41 @@ static __device__ __noinline__ double rcp_fp64_pipe(double x) {
 // units of the last place.  Measured per warp: latency 243 -> 148 clocks,
 // throughput 204 -> 48 clocks; FP64 solve of 59M compartments with the copy
 // of b 2.13 -> 1.92 ms, cable step of 14M 1.56 -> 1.35 ms.
-__device__ __forceinline__ double rcp_t(double x) {
+// In two halves, so that a caller can place FP64 instructions that do not
+// depend on it between them.
+struct RcpHalf {
+  double x;
+  float r, e1, p, pl;
+};
+__device__ __forceinline__ RcpHalf rcp_begin(double x) {
   const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-  // zero, subnormal, infinite, NaN, or a reciprocal below the normal range
-  if (((hi & 0x7FF00000u) - 0x00100000u) > (2043u << 20)) return rcp_fp64_pipe(x);
   const float xf = __uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7FFFFFu) | 0x3F800000u);
   const float x1 = __fmul_rn(__uint2float_rn(lo & 0x1FFFFFE0u), 0x1p-52f);
   const float x2 = __fmul_rn(__uint2float_rn(lo & 0x1Fu), 0x1p-52f);
   const float r = rcp_t(xf);
   const float e1 = __fmaf_rn(-xf, r, 1.f);  // exact
   const float p = __fmul_rn(x1, r), pl = __fmaf_rn(x2, r, __fmaf_rn(x1, r, -p));
-  const float s = __fsub_rn(e1, p), bb = __fsub_rn(s, e1);
-  const float el = __fsub_rn(__fsub_rn(__fsub_rn(e1, __fsub_rn(s, bb)), __fadd_rn(p, bb)), pl);
+  return {x, r, e1, p, pl};
+}
+__device__ __forceinline__ double rcp_end(const RcpHalf& c) {
+  const uint32_t hi = (uint32_t)__double2hiint(c.x);
+  // zero, subnormal, infinite, NaN, or a reciprocal below the normal range
+  if (((hi & 0x7FF00000u) - 0x00100000u) > (2043u << 20)) return rcp_fp64_pipe(c.x);
+  const float s = __fsub_rn(c.e1, c.p), bb = __fsub_rn(s, c.e1);
+  const float el = __fsub_rn(__fsub_rn(__fsub_rn(c.e1, __fsub_rn(s, bb)), __fadd_rn(c.p, bb)), c.pl);
   const float t = __fmaf_rn(s, s, el);  // e + e^2 = s + t
-  const float rs = __fmul_rn(r, 0x1p53f);
+  const float rs = __fmul_rn(c.r, 0x1p53f);
   constexpr float kBig = 0x1.8p32f, kOne = 0x1.8p23f;  // units of 512 and of 1
   const float a = __fmaf_rn(rs, s, kBig);
   const float b = __fadd_rn(__fmaf_rn(rs, t, __fmaf_rn(rs, s, -__fsub_rn(a, kBig))), kOne);
   const int32_t k = ((int32_t)__float_as_uint(a) - 0x4FC00000) * 512 + ((int32_t)__float_as_uint(b) - 0x4B400000);
-  const uint32_t rb = __float_as_uint(r);
+  const uint32_t rb = __float_as_uint(c.r);
   // r widened (exponent re-biased by 896, mantissa moved up by 29 bits), scaled by x's exponent, with x's sign
   const uint32_t oh = (rb >> 3) + (0x7FD00000u - 0x07E00000u) - (hi & 0xFFF00000u);
   const uint64_t o = ((uint64_t)oh << 32) | (uint64_t)(rb << 29);
   return __longlong_as_double((long long)(o + (uint64_t)(int64_t)k));
 }
+__device__ __forceinline__ double rcp_t(double x) { return rcp_end(rcp_begin(x)); }
 
 // ---- double-float arithmetic from FP32 error-free transformations -------------
 // A value is an unevaluated pair hi + lo; every product and sum below uses the

@@ -54,8 +54,6 @@ constexpr int teams_per_sm(int bytes, int most) {
   return kSmemPerSm / (bytes + 16 + 1024) < most ? kSmemPerSm / (bytes + 16 + 1024) : most;
 }
 
-constexpr int kAlwaysTeams = 1 << 30;
-
 template <int P>
 struct Geo {
   static constexpr int kChunk = 32 * P;              // pieces per chunk
@@ -392,9 +390,11 @@ struct CompMode {
   static constexpr int kTeamBytes = 2 * kStageBytes + kCacheBytes;
   static constexpr int kWarpBytes = kStageBytes + kCacheBytes;
   static constexpr int kMinBlocks = teams_per_sm(kTeamBytes, 12), kMinBlocksAlone = teams_per_sm(2 * kWarpBytes, 12);
-  // teams up to 18/16 entries per resident team (team against lone warp, us:
-  // 1940 entries 240 : 290, 1421 377 : 414, 2629 677 : 645, 2790 598 : 518)
-  static constexpr int kTeamShare = 18;
+  // teams in phase A up to this many sixteenths of an entry per resident team
+  // (team against lone warp, us a solve: 1940 entries 240 : 290, 1421 377 :
+  // 414; phase A alone, 2370 entries 535 : 573; solver layout, whose copies are
+  // bulk copies, 1197 381 : 412, 2629 665 : 601)
+  static constexpr int kTeamShare = kPk ? 18 : 24;
   static_assert(kStageBytes % 16 == 0, "16-byte aligned buffers");
   using Bulk = BulkStage<kTab + 80>;
 
@@ -683,11 +683,10 @@ struct FactorMode {
   static constexpr int kTeamBytes = 2 * kStageBytes + kCacheBytes;
   static constexpr int kWarpBytes = kStageBytes + kCacheBytes;
   static constexpr int kMinBlocks = teams_per_sm(kTeamBytes, 10), kMinBlocksAlone = teams_per_sm(2 * kWarpBytes, 10);
-  // teams up to this many sixteenths of an entry per resident team (team
-  // against lone warp, us; FP64: 1434 entries 262 : 318, 1940 668 : 764, 2340
-  // 655 : 633, 3760 560 : 535; FP32: 1940 195 : 236, 2629 558 : 479; re-using
-  // a factor: 2823 2511 : 2817, 2751 5731 : 5727)
-  static constexpr int kTeamShare = kReuse ? 40 : kYG ? 28 : 21;
+  // the same (us; FP64: 1434 entries 262 : 318, 1940 668 : 764, 2340 655 :
+  // 633, 3760 560 : 535; FP32: 1940 195 : 236, phase A alone, 2715 235 : 329;
+  // re-using a factor: 2823 2511 : 2817, 2751 5731 : 5727)
+  static constexpr int kTeamShare = kReuse ? 40 : kYG ? 28 : 32;
   // the factor block is staged by bulk copies
   static constexpr bool kBulk = kBF;
   static_assert(kStageBytes % 16 == 0, "16-byte aligned buffers");
@@ -924,31 +923,41 @@ struct FactorMode {
 #pragma unroll 1
         for (; c < q.nchild; ++c) child(c, make_double2(0.0, 0.0), false);
       }
-      // one row's factor from its pivot: g (or the multiplier) is returned
-      auto factor_row = [&](int h, int r, bool root) {
+      // a row's factor: FP64 (g, y) and, for later steps, the reciprocal;
+      // FP32 the reciprocal and the right-hand side (a root's x)
+      auto put_row = [&](int h, int r, T f, T y, T rr) {
         const int i = rows.slot(r, me + h);
-        const T rr = kReuse ? rk[h] : rcp_solve(kCable && !root ? D[h] - uk[h] : D[h]);
-        const T f = kReuse ? uk[h] : uk[h] * rr;
         if constexpr (kYG) {
-          const T y = B[h] * rr;
-          const T gs = root ? T(0) : f;  // a cell's root: x = y
           if constexpr (kBF) {
             const int q = tab[r] + me + h;
             if (kReuse)
               bf[q].y = y;
             else
-              bf[q] = make_double2(gs, y);
+              bf[q] = make_double2(f, y);
             if (keep_rcp) rcp_block[q] = rr;
           } else {
-            if (!kReuse) sd[i] = gs;
+            if (!kReuse) sd[i] = f;
             if (keep_rcp) su[i] = rr;
             sb[i] = y;
           }
         } else {
           sd[i] = rr;
-          sb[i] = root ? B[h] * rr : B[h];  // a root's x
+          sb[i] = y;
         }
-        return f;
+      };
+      // FP64: a row's y and the next right-hand side are left for the next
+      // row (late_part), where they fill the FP64 pipe while that row's
+      // reciprocal, which does not use it, is formed: the chain from pivot to
+      // pivot is then the reciprocal and two FP64 instructions.
+      constexpr bool kLate = kYG && !kReuse;
+      T fp[P], rp[P], bc[P];  // the row before: its factor and reciprocal; this row's right-hand side as given
+#pragma unroll
+      for (int h = 0; h < P; ++h) fp[h] = rp[h] = bc[h] = T(0);
+      auto late_part = [&](int h, int r) {  // of row r - 1
+        if (!kLate || r <= first_row[h]) return;
+        const T y = B[h] * rp[h];
+        B[h] = bc[h] - fp[h] * B[h];
+        put_row(h, r - 1, fp[h], y, rp[h]);
       };
       // rows from the distal end: the factor, then the chain to the next row
 #pragma unroll kUnroll
@@ -959,11 +968,23 @@ struct FactorMode {
             if (r < first_row[h]) continue;
             const int i1 = rows.slot(r + 1, me + h);
             const T a1 = sd[i1], b1 = sb[i1], u1 = su[i1];
-            const T f = factor_row(h, r, false);
-            if (!kReuse) D[h] = a1 - f * (kCable ? D[h] : uk[h]);
-            B[h] = b1 - f * B[h];
+            if constexpr (kLate) {
+              const RcpHalf half = rcp_begin(kCable ? D[h] - uk[h] : D[h]);
+              late_part(h, r);
+              rp[h] = rcp_end(half);
+              fp[h] = uk[h] * rp[h];
+              D[h] = a1 - fp[h] * (kCable ? D[h] : uk[h]);
+              bc[h] = b1;
+            } else {
+              const T rr = kReuse ? rk[h] : rcp_solve(D[h]);
+              const T f = kReuse ? uk[h] : uk[h] * rr;
+              if (!kReuse) D[h] = a1 - f * uk[h];
+              const T bn = b1 - f * B[h];
+              put_row(h, r, f, kYG ? B[h] * rr : B[h], rr);
+              B[h] = bn;
+              rk[h] = a1;
+            }
             uk[h] = u1;
-            rk[h] = a1;
           }
         }
       }
@@ -972,7 +993,10 @@ struct FactorMode {
       for (int h = 0; h < P; ++h) {
         if (m.p[h].len == 0) continue;
         const bool root = m.p[h].pcomp < 0;
-        const T f = factor_row(h, L - 1, root);
+        const T rr = kReuse ? rk[h] : rcp_solve(kCable && !root ? D[h] - uk[h] : D[h]);
+        late_part(h, L - 1);
+        const T f = root ? T(0) : kReuse ? uk[h] : uk[h] * rr;  // a cell's root: x = y
+        put_row(h, L - 1, f, kYG || root ? B[h] * rr : B[h], rr);
         const T cd = root || kReuse ? T(0) : f * (kCable ? D[h] : uk[h]), cb = root ? T(0) : f * B[h];
         const size_t pos = (size_t)(c0 + me + h);
         slot[2 * pos] = cd;
@@ -1124,10 +1148,11 @@ struct RefineMode {
   static constexpr int kStageBytes = kTab + 96;
   static constexpr int kCslot = 0, kCx = 0, kCacheBytes = 2 * G::kChunk * 16;
   static constexpr int kTeamBytes = 2 * kStageBytes + kCacheBytes;
-  static constexpr int kMinBlocks = teams_per_sm(kTeamBytes, 10);
-  // always teams (against lone warps, us: 700 entries 625 : 958, 2700 1610 :
-  // 2093): the copies outweigh the short arithmetic
-  static constexpr int kTeamShare = kAlwaysTeams;
+  static constexpr int kWarpBytes = kStageBytes + kCacheBytes;
+  static constexpr int kMinBlocks = teams_per_sm(kTeamBytes, 10), kMinBlocksAlone = teams_per_sm(2 * kWarpBytes, 10);
+  // the same, always (us a solve of one step: 700 entries 625 : 958, 2700 1610
+  // : 2093): the copies outweigh the short arithmetic
+  static constexpr int kTeamShare = 1 << 20;
   __device__ static void init_buffer(unsigned char*) {}
 
   // what the chunk needs of earlier chunks: the parent's x (visit 0), the
@@ -1529,21 +1554,11 @@ __device__ __forceinline__ int hand_over(const DevPlan& P, int t) {
 
 // kTeam: a CTA is one team; else its two warps run a task each.
 template <class M, bool kTeam>
-constexpr int min_blocks() {
-  if constexpr (kTeam)
-    return M::kMinBlocks;
-  else
-    return M::kMinBlocksAlone;
-}
-template <class M, bool kTeam>
 __host__ __device__ constexpr int cta_bytes() {
-  if constexpr (kTeam)
-    return M::kTeamBytes + 16;
-  else
-    return 2 * M::kWarpBytes;
+  return kTeam ? M::kTeamBytes + 16 : 2 * M::kWarpBytes;
 }
 template <class M, bool kTeam>
-__global__ void __launch_bounds__(64, min_blocks<M, kTeam>())
+__global__ void __launch_bounds__(64, kTeam ? M::kMinBlocks : M::kMinBlocksAlone)
     k_units(DevPlan P, typename M::Args A, int phase) {
   extern __shared__ __align__(16) unsigned char smem_u[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1612,9 +1627,7 @@ cudaError_t grid_of(const DevPlan& P, int* grid) {
 template <class M>
 cudaError_t grid_of(const DevPlan& P, int2* grid) {
   cudaError_t e = grid_of<M, true>(P, &grid->x);
-  if constexpr (M::kTeamShare != kAlwaysTeams)
-    if (e == cudaSuccess) e = grid_of<M, false>(P, &grid->y);
-  return e;
+  return e == cudaSuccess ? grid_of<M, false>(P, &grid->y) : e;
 }
 
 template <class M>
@@ -1623,11 +1636,16 @@ cudaError_t launch_phases(const DevPlan& P, const typename M::Args& A, int2 grid
   for (int phase = 0; phase < 3; ++phase) {
     const int ne = P.phase_off[phase + 1] - P.phase_off[phase];
     if (ne == 0) continue;
-    // teams where one runner per entry leaves the chip idle anyway, lone
-    // warps, twice as many tasks at a time, where there are entries for them
-    if (M::kTeamShare == kAlwaysTeams || ne <= M::kTeamShare * grid.x / 16) {
+    // Teams where one warp per entry leaves the chip idle anyway or a task's
+    // own latency decides, lone warps, twice as many tasks at a time, where
+    // there are entries for them.  Phase A ends with the top parts, one after
+    // the other's chunks: the mode's share.  Phase C (subtrees'
+    // substitutions) has no such tail: teams while every entry has one (2306
+    // entries on 1824 teams 263 us, on lone warps 214).
+    const int share = phase == 0 ? M::kTeamShare : 16;
+    if ((int64_t)ne * 16 <= (int64_t)share * grid.x) {
       k_units<M, true><<<ne < grid.x ? ne : grid.x, 64, cta_bytes<M, true>(), s>>>(P, A, phase);
-    } else if constexpr (M::kTeamShare != kAlwaysTeams) {
+    } else {
       const int ctas = (ne + 1) / 2;
       k_units<M, false><<<ctas < grid.y ? ctas : grid.y, 64, cta_bytes<M, false>(), s>>>(P, A, phase);
     }

@@ -31,8 +31,9 @@ def _batch(times, **opts):
     r = np.random.default_rng(4)
     probs = [problem(p, r) for p in trees]
     extra = [dict(g=r.uniform(0.1, 1.0, p.size), V=r.uniform(-80, -50, p.size)) for p in trees]
+    # (even cuts: aligned ones depend on where a cell starts in the batch)
     plan = H.Plan(np.tile([p.size for p in trees], times), np.tile(np.concatenate(trees), times),
-                  pack_compartments=1, **opts)
+                  pack_compartments=1, even_cuts=True, **opts)
     arrays = {k: np.concatenate([q[k] for q in probs]) for k in ("d", "u", "b", "s")}
     arrays.update({k: np.concatenate([q[k] for q in extra]) for k in ("g", "V")})
     return plan, {k: torch.as_tensor(np.tile(v, times)).cuda() for k, v in arrays.items()}
