@@ -556,6 +556,11 @@ struct CompMode {
     }
     FFV<V> X{vpack<P>(xph), vpack<P>(xpl)};
     float xbh = 0.f, xbl = 0.f;  // the second piece's distal solution
+    // a row's factor is read before the row above it writes its solution (the
+    // compiler may not move the read over the write)
+    float4 f[P];
+#pragma unroll
+    for (int h = 0; h < P; ++h) f[h] = sf[tab[L - 1] + me + h];
 #pragma unroll kUnroll
     for (int r = kL - 1; r >= 0; --r) {
       if (r < L) {
@@ -563,11 +568,11 @@ struct CompMode {
         float yh[P], yl[P], gh[P], gl[P];
 #pragma unroll
         for (int h = 0; h < P; ++h) {
-          const float4 f = sf[q + h];
-          yh[h] = f.x;
-          yl[h] = f.y;
-          gh[h] = f.z;
-          gl[h] = f.w;
+          yh[h] = f[h].x;
+          yl[h] = f[h].y;
+          gh[h] = f[h].z;
+          gl[h] = f[h].w;
+          if (r > 0) f[h] = sf[tab[r - 1] + me + h];
         }
         const FFV<V> gx = vmul_ff(FFV<V>{vpack<P>(gh), vpack<P>(gl)}, X);
         X = vsub_ffff(FFV<V>{vpack<P>(yh), vpack<P>(yl)}, gx.h, gx.l);
