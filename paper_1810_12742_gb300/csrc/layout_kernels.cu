@@ -26,7 +26,8 @@ namespace {
 // as many warps as shared memory holds work at once.  (As a visit of the
 // solves' task driver it walked every task twice, in two launches: 249 us for
 // 21M compartments of 8 bytes; a warp
-// per chunk 103 us; re-rooted plan 540, now 226 us.)
+// per chunk 103 us, with the next chunk's metadata on its way 93 us; re-rooted
+// plan 540, now 223 us.)
 //
 // (Packing stays slot by slot: a chunk-wise gather measured slower than the
 // plain kernel below, 1.02 against 0.66 ms per FP32 array of the full
@@ -55,13 +56,28 @@ __global__ void __launch_bounds__(32 * Unpack<W, P>::kWarps)
   W* sc = reinterpret_cast<W*>(buf + U::kRowBytes);
   if (lane == 0) U::Bulk::init(buf);
   __syncwarp();
-  for (int k = blockIdx.x * U::kWarps + w; k < Pl.n_chunks; k += gridDim.x * U::kWarps) {
-    const int c0 = __ldg(Pl.chunk_pos + k), n = __ldg(Pl.chunk_pos + k + 1) - c0;
-    const Meta<P> m = unpack_meta(load_meta<false, P>(Pl, c0, n, lane, true));
+  // a chunk's metadata is loaded while the chunk before it is moved
+  const int step = gridDim.x * U::kWarps;
+  int n_next = 0;
+  auto load = [&](int k) {
+    int c0 = 0;
+    n_next = 0;
+    if (k < Pl.n_chunks) {
+      c0 = __ldg(Pl.chunk_pos + k);
+      n_next = __ldg(Pl.chunk_pos + k + 1) - c0;
+    }
+    return load_meta<false, P>(Pl, c0, n_next, lane, true);
+  };
+  int k = blockIdx.x * U::kWarps + w;
+  RawMeta<false, P> r = load(k);
+  for (; k < Pl.n_chunks; k += step) {
+    const Meta<P> m = unpack_meta(r);
+    const int n = n_next;
     build_row_table<P>(m.L, lane, tab);
     // the block with its padding: blocks start on multiples of 4 slots, so
     // this is the distance to the next block (whole 16-byte words)
     U::Bulk::template issue<1>(buf, lane, (unsigned)(((tab[kL] + 3) & ~3) * (int)sizeof(W)), buf, src + m.blk);
+    r = load(k + step);
     U::Bulk::wait(Pl, buf, lane);
     for (int r = 0; r < m.L; ++r) {
       const int t = m.L - 1 - r;  // distance from the proximal end (pieces of a pair aligned there)
