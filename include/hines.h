@@ -111,7 +111,7 @@ typedef struct {
 typedef struct {
   int32_t n_cells;
   int32_t max_levels;       /* deepest branch dependency tree (levels of Section 3) */
-  int32_t n_tasks;          /* warp tasks: groups of cells solved together by one warp */
+  int32_t n_tasks;          /* warp tasks: groups of cells solved together by one warp (or team of two) */
   int32_t reserved;
   int64_t n_unknowns;       /* total compartments */
   int64_t n_branches;       /* unbranched runs after optional splitting */

@@ -80,7 +80,7 @@ struct HostPlan {
 
 constexpr int kLanes = 32;       // lanes of a warp; a chunk holds 32 * per_lane pieces
 constexpr int kBranchCap = 16;   // maximum compartments per branch after capping
-constexpr int kWarpsPerCta = 2;  // warps per CTA of the task kernels (each warp runs its own task)
+constexpr int kWarpsPerCta = 2;  // warps per CTA of the task kernels (one team, or a task each)
 constexpr int64_t kCutAlign = 8; // pieces of a cut branch start on multiples of 8 natural indices (32-byte sectors)
 constexpr int64_t kUnitMax = 4096;  // largest unit (compartments); larger cells are cut
 constexpr int64_t kPackAlign = 4;   // solver-layout blocks start on multiples of 4 compartments

@@ -1,13 +1,15 @@
 // Warp-task kernels of the batched Hines solver, sm_103a.
 //
 // The planner cuts every cell into units -- whole small cells, or the top part
-// and the subtrees of a large cell -- and packs units into tasks.  A team of
-// two warps owns a task and walks its chunks (Hu's list schedule of the task's
-// pieces, at most 32 * P pieces each, longest first): deepest chunk first for
-// the elimination, root-side chunk first for the substitution (Section 3).
-// One warp computes; the other moves data, so that copying a chunk's results
-// out and staging the next chunk's inputs overlap the arithmetic (run_task).
-// Lane j of the computing warp owns the chunk's pieces P j .. P j + P - 1 (P = 1 or 2 pieces per lane).
+// and the subtrees of a large cell -- and packs units into tasks.  A runner --
+// a team of two warps, or a lone warp in launches with many entries -- owns a
+// task and walks its chunks (Hu's list schedule of the task's pieces, at most
+// 32 * P pieces each, longest first): deepest chunk first for the
+// elimination, root-side chunk first for the substitution (Section 3).  In a
+// team one warp computes; the other moves data, so that copying a chunk's
+// results out and staging the next chunk's inputs overlap the arithmetic
+// (run_task).  Lane j of the computing warp owns the chunk's pieces P j ..
+// P j + P - 1 (P = 1 or 2 pieces per lane).
 // Inside a piece the parent of compartment i is i - 1 (Section 5): the lane
 // runs a Thomas chain (Listing 1) and leaves one contribution for its parent
 // compartment (Listing 2's parent lookup).  With P = 2 the lane runs its two
@@ -17,11 +19,11 @@
 // arithmetic runs on packed FP32-pair instructions.
 //
 // A solve is two launches: (A) whole-cell tasks (both sweeps), the
-// elimination of subtree tasks and, taken over by the team that finishes a
+// elimination of subtree tasks and, taken over by the runner that finishes a
 // cell's last subtree, that cell's top part (both sweeps); (C) the
-// substitution of subtree tasks.  No team ever waits for another.
+// substitution of subtree tasks.  No runner ever waits for another.
 //
-// The chunks of a task follow one another in the same team, so a chunk's
+// The chunks of a task follow one another in the same runner, so a chunk's
 // children are usually in the chunk just before it (elimination) and its
 // parents likewise (substitution): those values pass through a small shared
 // memory cache; other values go through global memory.  A chunk's inputs are
