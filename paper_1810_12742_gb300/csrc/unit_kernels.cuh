@@ -690,10 +690,11 @@ struct FactorMode {
   static constexpr int kTeamBytes = 2 * kStageBytes + kCacheBytes;
   static constexpr int kWarpBytes = kStageBytes + kCacheBytes;
   static constexpr int kMinBlocks = teams_per_sm(kTeamBytes, 10), kMinBlocksAlone = teams_per_sm(2 * kWarpBytes, 10);
-  // the same (us; FP64: 1434 entries 262 : 318, 1940 668 : 764, 2340 655 :
-  // 633, 3760 560 : 535; FP32: 1940 195 : 236, phase A alone, 2715 235 : 329;
-  // re-using a factor: 2823 2511 : 2817, 2751 5731 : 5727)
-  static constexpr int kTeamShare = kReuse ? 40 : kYG ? 28 : 32;
+  // the same (us; FP64: 1440 entries 262 : 318, 1514 668 : 764, 2184 376 :
+  // 392, 2260 586 : 628, 2707 542 : 509, 2755 954 : 953; FP32: 1514 195 : 236,
+  // phase A alone, 2715 235 : 329; re-using a factor: 2184 2511 : 2817, 2700
+  // 5731 : 5727)
+  static constexpr int kTeamShare = kReuse ? 40 : 32;
   // the factor block is staged by bulk copies
   static constexpr bool kBulk = kBF;
   static_assert(kStageBytes % 16 == 0, "16-byte aligned buffers");
