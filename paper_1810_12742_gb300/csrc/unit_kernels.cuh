@@ -1545,10 +1545,12 @@ __device__ void run_task_alone(const DevPlan& Pl, const typename M::Args& A, con
 // pending count; the team that finishes the cell's last subtree takes over
 // the cell's top part (both visits) as its next task, and restores the count
 // for the next call.  Nothing waits: the hand-over goes to whoever arrives
-// last.  Release: every lane fenced its writes before the team's last barrier;
-// acquire: the fence after the atomic, before the team's next barrier, and the
-// top part reads those slots through L2.  One thread; returns the top task, or
-// -1.
+// last.  One thread; returns the top task, or -1.  Release: every lane fenced
+// its writes before the team's last barrier (a lone warp's __syncwarp), which
+// this thread passed.  Acquire: this thread's fence after the atomic reaches
+// the other lanes of a team through the team's next barrier; a lone warp's
+// lanes, which learn of the top part by a shuffle (no memory ordering), fence
+// themselves (k_units).  The top part reads those slots through L2.
 __device__ __forceinline__ int hand_over(const DevPlan& P, int t) {
   const int cell = __ldg(P.task_sub + 2 * t);
   if (cell < 0) return -1;
@@ -1611,6 +1613,10 @@ __global__ void __launch_bounds__(64, kTeam ? M::kMinBlocks : M::kMinBlocksAlone
       __syncthreads();
     } else {
       k = __shfl_sync(kFull, k, 0);
+      if (k < 0) {  // a top part: every lane's side of the acquire (hand_over)
+        __threadfence();
+        __syncwarp();
+      }
     }
     if (k >= ne) break;
     t = k >= 0 ? entry(k) : TaskRec{(uint32_t)P.task_lvl_off[-2 - k], P.task_nlvl[-2 - k], -2 - k, 0};
