@@ -169,6 +169,10 @@ hines_status upload(hines_plan_t p) {
   D.n_unknowns = H.n_unknowns;
   D.n_branches = (int64_t)nb;
   if (hines::prepare_unit_kernels(D) != cudaSuccess) return HINES_ERR_CUDA;
+  // A copy from pageable memory returns once its bytes are staged, maybe before
+  // they are on the device, and streams that do not block on the legacy stream
+  // are not ordered after it: the plan is handed out only when all of it is there.
+  if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) return HINES_ERR_CUDA;
   return HINES_OK;
 }
 
