@@ -26,7 +26,8 @@
  * Asynchrony.  Calls that take a stream only enqueue work on it and return;
  * argument errors are returned synchronously, before anything is enqueued.
  * Calls that share a plan must be ordered on one stream (they share the
- * plan's workspace).  Nothing is allocated inside the solve calls.
+ * plan's workspace); the results of calls that are not are undefined, later
+ * ordered calls are sound.  Nothing is allocated inside the solve calls.
  *
  * Errors.  Every entry point returns a hines_status; hines_status_string
  * gives its text.  Device-side errors raise the plan's status word, read with
@@ -494,6 +495,18 @@ hines_status hines_pipeline_destroy(hines_pipeline_t pipeline);
  * faults or hangs, and the context stays usable afterwards.
  */
 hines_status hines_check_bounded_wait(int32_t polls, int32_t arrive, int32_t *status_out, int64_t *elapsed_ns);
+
+/*
+ * Check of the plan's work counters (no paper counterpart).  Between calls
+ * every counter a solve expects to find at 0 is 0; *off_count receives how many
+ * are not, after everything enqueued on the device has ended.  With disturb =
+ * 1 the work counters and those of the cells solved in parts are then set to
+ * 1, as calls that were not ordered (see "Asynchrony") may find them on the
+ * way: the result of the next solve or cable call that uses them is
+ * undefined, that call leaves them at 0 again, and the calls after it are
+ * sound.  Synchronous.
+ */
+hines_status hines_check_counts(hines_plan_t plan, int32_t disturb, int64_t *off_count);
 
 /* Static text of a status code. */
 const char *hines_status_string(int32_t status);

@@ -97,7 +97,7 @@ hines_status upload(hines_plan_t p) {
       {H.tchild.data(), H.tchild.size() * 4, (const void**)&D.tchild},
       {phase_rec.data(), phase_rec.size() * sizeof(int4), (const void**)&D.phase_rec},
       {H.cell_top_task.data(), H.cell_top_task.size() * 4, (const void**)&D.cell_top_task},
-      {H.counter_init.data(), H.counter_init.size() * 4, (const void**)&D.counter_init},
+      {H.cell_nsub.data(), H.cell_nsub.size() * 4, (const void**)&D.cell_nsub},
       {H.task_sub.data(), H.task_sub.size() * 4, (const void**)&D.task_sub},
       {H.torder.data(), H.torder.size() * 4, (const void**)&D.pos_branch},
       {H.cell_off.data(), H.cell_off.size() * 8, (const void**)&D.cell_off},
@@ -154,10 +154,9 @@ hines_status upload(hines_plan_t p) {
   D.red = w;
   w += red_b;
   D.counter = reinterpret_cast<int32_t*>(w);
-  D.cell_pending = D.counter + 4;
+  D.cell_done = D.counter + 4;
   w += cnt_b;
-  if (cudaMemcpy(D.counter, H.counter_init.data(), H.counter_init.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess)
-    return HINES_ERR_CUDA;
+  if (cudaMemset(D.counter, 0, (nc + 4) * 4) != cudaSuccess) return HINES_ERR_CUDA;
   D.rw = w;
   w += rw_b;
   D.ff4 = w;
@@ -534,6 +533,33 @@ hines_status hines_plan_status(hines_plan_t p, int32_t* status_out) {
   if (cudaMemcpy(status_out, p->dev.status, sizeof(int32_t), cudaMemcpyDeviceToHost) != cudaSuccess)
     return HINES_ERR_CUDA;
   if (cudaMemset(p->dev.status, 0, sizeof(int32_t)) != cudaSuccess) return HINES_ERR_CUDA;
+  return HINES_OK;
+}
+
+hines_status hines_check_counts(hines_plan_t p, int32_t disturb, int64_t* off_count) {
+  const hines_status st = check_plan(p);
+  if (st != HINES_OK) return st;
+  if ((disturb != 0 && disturb != 1) || !off_count) return HINES_ERR_INVALID_ARG;
+  try {
+    std::vector<int32_t> counts((size_t)p->host.n_cells + 4);
+    const size_t bytes = counts.size() * sizeof(int32_t);
+    if (cudaDeviceSynchronize() != cudaSuccess ||
+        cudaMemcpy(counts.data(), p->dev.counter, bytes, cudaMemcpyDeviceToHost) != cudaSuccess)
+      return HINES_ERR_CUDA;
+    const int64_t zeros = std::count(counts.begin(), counts.end(), 0);
+    // (phase C's counter is zeroed by the launch before it in the same call)
+    *off_count = (int64_t)counts.size() - zeros - (counts[2] != 0 ? 1 : 0);
+    if (disturb) {
+      counts.assign(counts.size(), 0);
+      counts[0] = counts[2] = 1;
+      for (size_t c = 0; c + 4 < counts.size(); ++c) counts[c + 4] = p->host.cell_nsub[c] > 0 ? 1 : 0;
+      if (cudaMemcpy(p->dev.counter, counts.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
+          cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
+        return HINES_ERR_CUDA;
+    }
+  } catch (const std::bad_alloc&) {
+    return HINES_ERR_OOM;
+  }
   return HINES_OK;
 }
 

@@ -49,12 +49,13 @@ struct DevPlan {
   const int32_t* tchild = nullptr;        // child positions (non-contiguous children)
   const int4* phase_rec = nullptr;        // work entries, phases A, B (empty), C concatenated: the words of a TaskRec
   int32_t phase_off[4] = {0, 0, 0, 0};
-  int32_t* counter = nullptr;             // [4 + n_cells] work counters, then cell_pending (workspace)
-  const int32_t* counter_init = nullptr;  // [4 + n_cells] their values between calls (each launch restores them)
+  int32_t* counter = nullptr;             // [4 + n_cells] work counters by phase, then cell_done (workspace); all
+                                          // but phase C's, which phase A zeroes, 0 between calls (launch_phases)
+  const int32_t* cell_nsub = nullptr;     // [n_cells] subtree units of the cell
   const int32_t* cell_top_task = nullptr; // [n_cells] task of the cell's top part, -1 if not cut
   const int32_t* task_sub = nullptr;      // [2 * n_wtasks] (cell, subtree units) of a subtree task
   const int32_t* pos_branch = nullptr;    // [nb] branch id (natural numbering) of each position
-  int32_t* cell_pending = nullptr;        // counter + 4: subtree units whose elimination is still to finish
+  int32_t* cell_done = nullptr;           // counter + 4: subtree units whose elimination is finished
   // solver layout (Section 5's interleaving per chunk)
   int64_t n_packed = 0;
   int32_t n_chunks = 0;

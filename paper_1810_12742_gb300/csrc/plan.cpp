@@ -475,8 +475,6 @@ int build_host_plan(int32_t n_cells, const int32_t* ncomp, const int32_t* parent
   P.cell_nsub.assign((size_t)n_cells, 0);
   for (const auto& u : units)
     if (u.kind == 1) P.cell_nsub[(size_t)u.cell]++;
-  P.counter_init.assign(4, 0);
-  P.counter_init.insert(P.counter_init.end(), P.cell_nsub.begin(), P.cell_nsub.end());
   for (int64_t b = 0; b < nb; ++b)
     if (P.br_kind[(size_t)b] == 2) P.cell_top_task[(size_t)P.br_cell[(size_t)b]] = P.br_task[(size_t)b];
   // per task the cell its subtree units belong to (subtree tasks hold one

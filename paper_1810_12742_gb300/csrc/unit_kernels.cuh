@@ -1541,11 +1541,10 @@ __device__ void run_task_alone(const DevPlan& Pl, const typename M::Args& A, con
   __syncwarp();
 }
 
-// After a subtree task's elimination: count its units off their cell's
-// pending count; the team that finishes the cell's last subtree takes over
-// the cell's top part (both visits) as its next task, and restores the count
-// for the next call.  Nothing waits: the hand-over goes to whoever arrives
-// last.  One thread; returns the top task, or -1.  Release: every lane fenced
+// After a subtree task's elimination: count its units as done; whoever
+// finishes the cell's last subtree takes over the cell's top part (both
+// visits) as its next task.  Nothing waits: the hand-over goes to whoever
+// arrives last.  One thread; returns the top task, or -1.  Release: every lane fenced
 // its writes before the team's last barrier (a lone warp's __syncwarp), which
 // this thread passed.  Acquire: this thread's fence after the atomic reaches
 // the other lanes of a team through the team's next barrier; a lone warp's
@@ -1556,8 +1555,8 @@ __device__ __forceinline__ int hand_over(const DevPlan& P, int t) {
   if (cell < 0) return -1;
   const int cnt = __ldg(P.task_sub + 2 * t + 1);
   __threadfence();
-  if (atomicSub(P.cell_pending + cell, cnt) != cnt) return -1;
-  P.cell_pending[cell] = __ldg(P.counter_init + 4 + cell);
+  if (atomicAdd(P.cell_done + cell, cnt) + cnt != __ldg(P.cell_nsub + cell)) return -1;
+  P.counter[2] = 0;  // (phase C's, launch_phases)
   __threadfence();
   return __ldg(P.cell_top_task + cell);
 }
@@ -1594,9 +1593,8 @@ __global__ void __launch_bounds__(64, kTeam ? M::kMinBlocks : M::kMinBlocksAlone
   // the first entry of a runner (team or warp) is its own number, the others
   // are counted off
   int k = kTeam ? (int)blockIdx.x : 2 * (int)blockIdx.x + w;
-  if (k >= ne) return;  // (one warp of the last CTA, at most)
-  TaskRec t = entry(k);
-  for (;;) {
+  TaskRec t = entry(k < ne ? k : 0);
+  while (k < ne) {  // (one warp of the last CTA, at most, has no entry)
     if constexpr (kTeam)
       run_task<M>(P, A, t, mover, lane, smem);
     else
@@ -1621,9 +1619,10 @@ __global__ void __launch_bounds__(64, kTeam ? M::kMinBlocks : M::kMinBlocksAlone
     if (k >= ne) break;
     t = k >= 0 ? entry(k) : TaskRec{(uint32_t)P.task_lvl_off[-2 - k], P.task_nlvl[-2 - k], -2 - k, 0};
   }
-  // every runner ends on one count past the entries: the last of them restores
-  // the counter, so that no copy has to before the next call
-  if (lane == 0 && !mover && ne > runners && k == ne + runners - 1) *next_entry = 0;
+  if (phase == 2) {  // phase A's counts back to 0 (launch_phases)
+    if (blockIdx.x == 0 && threadIdx.x == 0) P.counter[0] = 0;
+    for (int c = blockIdx.x * 64 + threadIdx.x; c < P.n_cells; c += gridDim.x * 64) P.cell_done[c] = 0;
+  }
 }
 
 template <class M, bool kTeam>
@@ -1644,12 +1643,25 @@ cudaError_t grid_of(const DevPlan& P, int2* grid) {
   return e == cudaSuccess ? grid_of<M, false>(P, &grid->y) : e;
 }
 
+// The work counters and the cells' counts of finished subtrees are 0 when they
+// are needed without a copy before each call: phase C's launch zeroes phase
+// A's counter and every cell's count for the next call, phase A's hand-overs
+// zero phase C's counter, whatever they hold.  Where no cell is cut there is no phase C, and a memset follows phase A
+// if it counted entries off at all (FP64 solve of 59M compartments 1541.7 us
+// with and without).
+// So even calls that share a plan unordered, against the interface, leave sound
+// counts once they have all ended: each call's zeroing comes after its own
+// counting, hence the last zeroing after all of it.  (Restored by whoever drew
+// the last entry or finished the last subtree, a count that once went wrong
+// stayed wrong, and later calls left out entries or top parts silently.)
 template <class M>
 cudaError_t launch_phases(const DevPlan& P, const typename M::Args& A, int2 grid, cudaStream_t s) {
   if (P.n_wtasks == 0) return cudaSuccess;
+  const bool cut = P.phase_off[3] > P.phase_off[2];
   for (int phase = 0; phase < 3; ++phase) {
     const int ne = P.phase_off[phase + 1] - P.phase_off[phase];
     if (ne == 0) continue;
+    int runners;
     // Teams where one warp per entry leaves the chip idle anyway or a task's
     // own latency decides, lone warps, twice as many tasks at a time, where
     // there are entries for them.  Phase A ends with the top parts, one after
@@ -1658,13 +1670,19 @@ cudaError_t launch_phases(const DevPlan& P, const typename M::Args& A, int2 grid
     // entries on 1824 teams 263 us, on lone warps 214).
     const int share = phase == 0 ? M::kTeamShare : 16;
     if ((int64_t)ne * 16 <= (int64_t)share * grid.x) {
-      k_units<M, true><<<ne < grid.x ? ne : grid.x, 64, cta_bytes<M, true>(), s>>>(P, A, phase);
+      runners = ne < grid.x ? ne : grid.x;
+      k_units<M, true><<<runners, 64, cta_bytes<M, true>(), s>>>(P, A, phase);
     } else {
-      const int ctas = (ne + 1) / 2;
-      k_units<M, false><<<ctas < grid.y ? ctas : grid.y, 64, cta_bytes<M, false>(), s>>>(P, A, phase);
+      const int ctas = (ne + 1) / 2 < grid.y ? (ne + 1) / 2 : grid.y;
+      runners = 2 * ctas;
+      k_units<M, false><<<ctas, 64, cta_bytes<M, false>(), s>>>(P, A, phase);
     }
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && !cut && ne > runners) e = cudaMemsetAsync(P.counter, 0, 4 * sizeof(int32_t), s);
+    if (e != cudaSuccess) {
+      cudaMemsetAsync(P.counter, 0, ((size_t)P.n_cells + 4) * sizeof(int32_t), s);
+      return e;
+    }
   }
   return cudaSuccess;
 }

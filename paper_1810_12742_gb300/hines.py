@@ -39,7 +39,7 @@ EXPORTS = [
     "hines_cable_step_packed", "hines_cable_solve_packed", "hines_cable_step_reuse",
     "hines_pack_coupling", "hines_plan_export_reroot",
     "hines_pipeline_create", "hines_pipeline_info", "hines_pipeline_solve_compensated", "hines_pipeline_status",
-    "hines_pipeline_destroy", "hines_check_bounded_wait",
+    "hines_pipeline_destroy", "hines_check_bounded_wait", "hines_check_counts",
 ]
 
 
@@ -106,6 +106,7 @@ def lib():
             L.hines_pipeline_status.argtypes = [vp, vp]
             L.hines_pipeline_destroy.argtypes = [vp]
             L.hines_check_bounded_wait.argtypes = [i32, i32, vp, vp]
+            L.hines_check_counts.argtypes = [vp, i32, vp]
             L.hines_status_string.restype = ctypes.c_char_p
             for name in EXPORTS:
                 if name != "hines_status_string":
@@ -524,6 +525,14 @@ def check_bounded_wait(polls: int, arrive: bool = False):
     _check(lib().hines_check_bounded_wait(int(polls), int(bool(arrive)), ctypes.byref(st), ctypes.byref(ns)),
            "hines_check_bounded_wait")
     return st.value, ns.value
+
+
+def check_counts(plan: Plan, disturb: bool = False) -> int:
+    """hines_check_counts: how many of the plan's work counters are not 0
+    (none, between calls); disturb then sets them to 1."""
+    off = ctypes.c_int64()
+    _check(lib().hines_check_counts(plan.handle, int(bool(disturb)), ctypes.byref(off)), "hines_check_counts")
+    return off.value
 
 
 def _hptr(t, dtype, n, name):
