@@ -622,8 +622,8 @@ struct CompMode {
 // plan's factor block, 16 bytes in the chunk's block order of the solver
 // layout (each row a contiguous run), staged back with bulk copies, or to
 // natural (or slot) positions, g into the workspace and y in place.  A full
-// cable step also leaves the reciprocal pivot, which steps that re-use the
-// factor need for y.  FP32: the reciprocal pivot goes to the workspace and the
+// cable step or cable solve also leaves the reciprocal pivot, which steps that
+// re-use the factor need for y.  FP32: the reciprocal pivot goes to the workspace and the
 // right-hand side in place (the refinement reads that factor); the
 // substitution reads them and u back.  In cable mode
 // the system is rebuilt while staging (Section 1's implicit-Euler system):
@@ -680,7 +680,7 @@ struct FactorMode {
     const T* g;
     T* x;        // right-hand side in, solution out (cable: V in, V out)
     T dt, E, theta;
-    bool rhs_from_V;  // cable: a time step (else a solve with the step's matrix, which leaves no reciprocals)
+    bool rhs_from_V;  // cable: a time step (else a solve with the step's matrix)
     const T* rhs = nullptr;  // non-null: the right-hand side is read from here (x receives the solution)
   };
   // a staging buffer: d (or the factor), u, b, then the row table (solver layout)
@@ -704,9 +704,9 @@ struct FactorMode {
   }
   // (g, y) per slot of the solver layout
   __device__ static double2* factor_block(const DevPlan& Pl) { return static_cast<double2*>(Pl.ff4); }
-  // the reciprocal pivots of the last full step: the workspace the other placement's factor would use
+  // the reciprocal pivots of the last full elimination: the workspace the other placement's factor would use
   __device__ static T* reciprocals(const DevPlan& Pl) { return static_cast<T*>(kBF ? Pl.fac : Pl.ff4); }
-  __device__ static bool keeps_rcp(const Args& A) { return kYG && kCable && !kReuse && A.rhs_from_V; }
+  static constexpr bool kKeepRcp = kYG && kCable && !kReuse;
 
   // Section 1's implicit-Euler system, each part in the fewest operations: the
   // diagonal less all its edges, s (1 + theta dt g), and the right-hand side
@@ -889,7 +889,6 @@ struct FactorMode {
 #pragma unroll
     for (int h = 0; h < P; ++h) first_row[h] = m.p[h].len > 0 ? L - m.p[h].len : kL;
     if (visit == 0) {
-      const bool keep_rcp = keeps_rcp(A);
       T* rcp_block = kBF ? reciprocals(Pl) + m.blk : nullptr;
       // per piece: the eliminated pivot (cable: E) and right-hand side of the
       // current row, its coupling (re-using a factor: its g) and stored
@@ -942,10 +941,10 @@ struct FactorMode {
               bf[q].y = y;
             else
               bf[q] = make_double2(f, y);
-            if (keep_rcp) rcp_block[q] = rr;
+            if (kKeepRcp) rcp_block[q] = rr;
           } else {
             if (!kReuse) sd[i] = f;
-            if (keep_rcp) su[i] = rr;
+            if (kKeepRcp) su[i] = rr;
             sb[i] = y;
           }
         } else {
@@ -1099,7 +1098,7 @@ struct FactorMode {
     }
     T* fac = static_cast<T*>(Pl.fac);
     T* rc = reciprocals(Pl);
-    const bool keep_fac = visit == 0 && !kReuse, keep_rcp = visit == 0 && keeps_rcp(A);
+    const bool keep_fac = visit == 0 && !kReuse, keep_rcp = visit == 0 && kKeepRcp;
     if (kPk) {
       const int e = tab[kL];
 #pragma unroll 1

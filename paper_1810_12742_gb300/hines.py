@@ -374,7 +374,8 @@ def cable_step_packed(plan: Plan, s, g, u, V, dt: float, E: float, theta: int = 
 
 def cable_step_reuse(plan: Plan, s, g, u, V, dt: float, E: float, theta: int = 1, solver_layout: bool = False):
     """hines_cable_step_reuse: a cable step with the factor of the last full
-    step on this plan (same s, g, u, dt, theta and layout); V in place."""
+    cable step or cable solve on this plan (same s, g, u, dt, theta and layout);
+    V in place."""
     torch = _torch()
     n = plan.n_packed if solver_layout else plan.n_unknowns
     ptr = _pptr if solver_layout else _dptr
