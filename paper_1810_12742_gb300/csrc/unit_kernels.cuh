@@ -37,6 +37,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "../../include/hines.h"
 #include "device_common.cuh"
@@ -110,8 +111,8 @@ struct Meta {
   // predecessor left it, fetched a chunk ahead (fetch) so that its latency
   // overlaps the computation
   PreX xpre[P];
-  // elimination (FP64): the contributions of the first two children, where
-  // other chunks than the cached predecessor left them, fetched likewise
+  // elimination (factor modes): the contributions of the first two children,
+  // where other chunks than the cached predecessor left them, fetched likewise
   double2 cpre[P][2];
   int L;         // rows of the lane: length of its first (longer) piece, 0 for a lane without pieces
 };
@@ -184,6 +185,34 @@ __device__ __forceinline__ int child_pos(const DevPlan& Pl, const Piece& q, int 
   if (c == 0) return q.child0;
   if (q.nchild == 2) return q.child1;
   return q.ccontig ? q.child0 + c : __ldg(Pl.tchild + q.child1 + c);
+}
+
+// apply(load(c)) for the children of each lane's piece from child c on, in
+// order.  In a lone warp's kernel (kAlone) the lanes of `live`, the callers,
+// go in step, two children at a time: left to their own trip counts the lanes
+// of the FP32 kernels stayed apart after the loop and ran the rows behind it in
+// groups (FP32 solve of 1000 cells of 2000 compartments: 104 million warp
+// instructions with 13 threads each, 392 us; in step 60 with 18, 198 us).  The
+// teams' kernels do not, and lose 3 to 7% to the votes.
+template <bool kAlone, typename Load, typename Apply>
+__device__ __forceinline__ void for_children(unsigned live, int nchild, int c, Load&& load, Apply&& apply) {
+  if constexpr (kAlone) {
+#pragma unroll 1
+    for (; __any_sync(live, c < nchild); c += 2) {
+      if (c >= nchild) continue;
+      const auto a = load(c);
+      if (c + 1 < nchild) {
+        const auto b = load(c + 1);
+        apply(a);
+        apply(b);
+      } else {
+        apply(a);
+      }
+    }
+  } else {
+#pragma unroll 1
+    for (; c < nchild; ++c) apply(load(c));
+  }
 }
 
 // A child's contribution slot: through L2 when another warp may have written
@@ -405,6 +434,7 @@ struct CompMode {
     if (kBulk) Bulk::init(buf);
   }
   // what the chunk needs of earlier chunks that no cache holds
+  template <bool kAlone>
   __device__ static void fetch(const DevPlan& Pl, const Args&, int visit, Meta<P>& m, const Prev& pv) {
     if (visit == 0) return;
 #pragma unroll
@@ -456,6 +486,7 @@ struct CompMode {
     cp_commit();
   }
 
+  template <bool kAlone>
   __device__ static void compute(const DevPlan& Pl, const Args&, int visit, int c0, int n, int lane,
                                  const Meta<P>& m, unsigned char* buf, const Prev& pv, unsigned char* cache, int cur) {
     float4* cslot = reinterpret_cast<float4*>(cache + kCslot);  // [2][kChunk] contributions
@@ -465,6 +496,7 @@ struct CompMode {
     float2* xlast = static_cast<float2*>(Pl.xlast);
     if (bulk_staged(visit)) Bulk::wait(Pl, buf, lane);
     const int L = m.L;
+    const unsigned live = kAlone ? __ballot_sync(kFull, L > 0) : 0u;  // (for_children)
     if (L == 0) return;
     const int me = P * lane;
     // the second piece's distal row (it joins the chain there); L: none
@@ -481,17 +513,20 @@ struct CompMode {
         const Piece& q = m.p[h];
         d0h[h] = 1.f;
         d0l[h] = b0h[h] = b0l[h] = 0.f;
-        if (q.len == 0) continue;
-        const int idx = rows.slot(L - q.len, me + h);
-        ff Dv = {sd[idx], 0.f}, Bv = {sb[idx], 0.f};
-#pragma unroll 1
-        for (int c = 0; c < q.nchild; ++c) {
-          const int cp = child_pos(Pl, q, c);
-          const int loc = cp - pv.c0;
-          const float4 v = (loc >= 0 && loc < pv.n) ? cslot[pv.which * G::kChunk + loc] : slot_load(slot + cp, q);
-          Dv = ff_sub(Dv, v.x, v.y);
-          Bv = ff_sub(Bv, v.z, v.w);
-        }
+        if (!kAlone && q.len == 0) continue;  // (a lone warp's lanes go on together)
+        const int idx = q.len > 0 ? rows.slot(L - q.len, me + h) : 0;
+        ff Dv = {q.len > 0 ? sd[idx] : 1.f, 0.f}, Bv = {q.len > 0 ? sb[idx] : 0.f, 0.f};
+        for_children<kAlone>(
+            live, q.nchild, 0,
+            [&](int c) {
+              const int cp = child_pos(Pl, q, c);
+              const int loc = cp - pv.c0;
+              return (loc >= 0 && loc < pv.n) ? cslot[pv.which * G::kChunk + loc] : slot_load(slot + cp, q);
+            },
+            [&](const float4& v) {
+              Dv = ff_sub(Dv, v.x, v.y);
+              Bv = ff_sub(Bv, v.z, v.w);
+            });
         d0h[h] = Dv.h;
         d0l[h] = Dv.l;
         b0h[h] = Bv.h;
@@ -779,7 +814,14 @@ struct FactorMode {
   // or from the slots.
   __device__ static bool local_child(int cp, const Prev& pv) { return cp >= pv.c0 && cp < pv.c0 + pv.n; }
   // what the chunk needs of earlier chunks that no cache holds: a parent's
-  // solution, the contributions of the first two children
+  // solution, the contributions of the first two children (FP32: in lone
+  // warps, whose solver-layout kernel takes 148 us with it and 260 without on
+  // 1000 cells of 2000 compartments; teams gain nothing)
+  template <bool kAlone>
+  __device__ static constexpr bool fetches_children() {
+    return kYG || kAlone;
+  }
+  template <bool kAlone>
   __device__ static void fetch(const DevPlan& Pl, const Args&, int visit, Meta<P>& m, const Prev& pv) {
 #pragma unroll
     for (int h = 0; h < P; ++h) {
@@ -788,13 +830,16 @@ struct FactorMode {
         const int loc = q.ppos - pv.c0;
         if (q.len > 0 && q.pcomp >= 0 && !(loc >= 0 && loc < pv.n))
           pre_set(m.xpre[h], static_cast<const T*>(Pl.xlast)[q.ppos]);
-      } else if (kYG) {
-        const double2* slot = static_cast<const double2*>(Pl.cd);
+      } else if (fetches_children<kAlone>()) {
+        using T2 = std::conditional_t<kYG, double2, float2>;
+        const T2* slot = static_cast<const T2*>(Pl.cd);
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
           if (c >= q.nchild) continue;
           const int cp = child_pos(Pl, q, c);
-          if (!local_child(cp, pv)) m.cpre[h][c] = slot_load(slot + cp, q);
+          if (local_child(cp, pv)) continue;
+          const T2 v = slot_load(slot + cp, q);
+          m.cpre[h][c] = make_double2(v.x, v.y);
         }
       }
     }
@@ -870,6 +915,7 @@ struct FactorMode {
     cp_commit();
   }
 
+  template <bool kAlone>
   __device__ static void compute(const DevPlan& Pl, const Args& A, int visit, int c0, int n, int lane,
                                  const Meta<P>& m, unsigned char* buf, const Prev& pv, unsigned char* cache, int cur) {
     T* sd = reinterpret_cast<T*>(buf);
@@ -882,6 +928,7 @@ struct FactorMode {
     const Rows<kPk, P> rows{tab};
     if (kBulk && visit == 1) Bulk::wait(Pl, buf, lane);
     const int L = m.L;
+    const unsigned live = kAlone ? __ballot_sync(kFull, L > 0) : 0u;  // (for_children)
     if (L == 0) return;
     const int me = P * lane;
     double2* bf = kBF ? factor_block(Pl) + m.blk : nullptr;  // the chunk's factor block
@@ -899,36 +946,43 @@ struct FactorMode {
         const Piece& q = m.p[h];
         D[h] = T(1);
         B[h] = uk[h] = rk[h] = T(0);
-        if (q.len == 0) continue;
-        const int idx = rows.slot(first_row[h], me + h);
-        (kReuse ? rk[h] : D[h]) = sd[idx];
-        B[h] = sb[idx];
-        uk[h] = su[idx];
-        auto child = [&](int c, double2 pre, bool fetched) {
+        if (!kAlone && q.len == 0) continue;  // (a lone warp's lanes go on together)
+        if (q.len > 0) {
+          const int idx = rows.slot(first_row[h], me + h);
+          (kReuse ? rk[h] : D[h]) = sd[idx];
+          B[h] = sb[idx];
+          uk[h] = su[idx];
+        }
+        struct Contribution {
+          T cd, cb;
+        };
+        auto load = [&](int c, double2 pre, bool fetched) {
           const int cp = child_pos(Pl, q, c);
           const int w = (pv.which * G::kChunk + cp - pv.c0) * 2;
-          T cd, cb;
+          Contribution v;
           if (local_child(cp, pv)) {
-            cd = kReuse ? T(0) : cslot[w];
-            cb = cslot[w + 1];
+            v.cd = kReuse ? T(0) : cslot[w];
+            v.cb = cslot[w + 1];
           } else if (fetched) {
-            cd = (T)pre.x;
-            cb = (T)pre.y;
+            v.cd = (T)pre.x;
+            v.cb = (T)pre.y;
           } else {
-            cd = kReuse ? T(0) : slot_load(slot + 2 * (size_t)cp, q);
-            cb = slot_load(slot + 2 * (size_t)cp + 1, q);
+            v.cd = kReuse ? T(0) : slot_load(slot + 2 * (size_t)cp, q);
+            v.cb = slot_load(slot + 2 * (size_t)cp + 1, q);
           }
-          if (!kReuse) D[h] -= cd;
-          B[h] -= cb;
+          return v;
         };
-        int c = 0;
-        if (kYG) {
-          if (q.nchild > 0) child(0, m.cpre[h][0], true);
-          if (q.nchild > 1) child(1, m.cpre[h][1], true);
-          c = 2;
+        auto apply = [&](const Contribution& v) {
+          if (!kReuse) D[h] -= v.cd;
+          B[h] -= v.cb;
+        };
+        constexpr bool kPre = fetches_children<kAlone>();
+        if (kPre) {
+          if (q.nchild > 0) apply(load(0, m.cpre[h][0], true));
+          if (q.nchild > 1) apply(load(1, m.cpre[h][1], true));
         }
-#pragma unroll 1
-        for (; c < q.nchild; ++c) child(c, make_double2(0.0, 0.0), false);
+        for_children<kAlone>(
+            live, q.nchild, kPre ? 2 : 0, [&](int c) { return load(c, make_double2(0.0, 0.0), false); }, apply);
       }
       // a row's factor: FP64 (g, y) and, for later steps, the reciprocal;
       // FP32 the reciprocal and the right-hand side (a root's x)
@@ -1164,6 +1218,7 @@ struct RefineMode {
 
   // what the chunk needs of earlier chunks: the parent's x (visit 0), the
   // parent's correction where no cache holds it (visit 1)
+  template <bool kAlone>
   __device__ static void fetch(const DevPlan& Pl, const Args& A, int visit, Meta<P>& m, const Prev& pv) {
 #pragma unroll
     for (int h = 0; h < P; ++h) {
@@ -1228,6 +1283,7 @@ struct RefineMode {
     s = s1;
   }
 
+  template <bool kAlone>
   __device__ static void compute(const DevPlan& Pl, const Args& A, int visit, int c0, int n, int lane,
                                  const Meta<P>& m, unsigned char* buf, const Prev& pv, unsigned char* cache, int cur) {
     float* sd = reinterpret_cast<float*>(buf);
@@ -1240,6 +1296,7 @@ struct RefineMode {
     float4* slot = static_cast<float4*>(Pl.cd);
     float2* xlast = static_cast<float2*>(Pl.xlast);
     const int L = m.L;
+    const unsigned live = kAlone ? __ballot_sync(kFull, L > 0) : 0u;  // (for_children)
     if (L == 0) return;
     const int me = P * lane;
     const int delta = P == 2 ? L - m.p[P - 1].len : 0;
@@ -1254,21 +1311,24 @@ struct RefineMode {
       for (int h = 0; h < P; ++h) {
         const Piece& q = m.p[h];
         xph[h] = xpl[h] = crh[h] = crl[h] = ce[h] = 0.f;
-        if (q.len == 0) continue;
-        if (q.pcomp >= 0) {
+        if (!kAlone && q.len == 0) continue;  // (a lone warp's lanes go on together)
+        if (q.len > 0 && q.pcomp >= 0) {
           const float2 t = m.xpre[h].ff;
           xph[h] = t.x;
           xpl[h] = t.y;
         }
         ff acc = {0.f, 0.f};
-#pragma unroll 1
-        for (int c = 0; c < q.nchild; ++c) {
-          const int cp = child_pos(Pl, q, c);
-          const int loc = cp - pv.c0;
-          const float4 v = (loc >= 0 && loc < pv.n) ? cslot[pv.which * G::kChunk + loc] : slot_load(slot + cp, q);
-          acc = ff_sub(acc, -v.x, -v.y);
-          ce[h] += v.z;
-        }
+        for_children<kAlone>(
+            live, q.nchild, 0,
+            [&](int c) {
+              const int cp = child_pos(Pl, q, c);
+              const int loc = cp - pv.c0;
+              return (loc >= 0 && loc < pv.n) ? cslot[pv.which * G::kChunk + loc] : slot_load(slot + cp, q);
+            },
+            [&](const float4& v) {
+              acc = ff_sub(acc, -v.x, -v.y);
+              ce[h] += v.z;
+            });
         crh[h] = acc.h;
         crl[h] = acc.l;
       }
@@ -1454,7 +1514,7 @@ __device__ void run_task(const DevPlan& Pl, const typename M::Args& A, const Tas
   if (mover)
     stage(cur, m_cur, 0);
   else
-    M::fetch(Pl, A, cur.visit, m_cur, pv);
+    M::template fetch<false>(Pl, A, cur.visit, m_cur, pv);
   Meta<P> m_nxt = unpack_meta(r_nxt);
   int which = 0;
   __syncthreads();
@@ -1468,8 +1528,8 @@ __device__ void run_task(const DevPlan& Pl, const typename M::Args& A, const Tas
       __syncwarp();
       if (!turn) stage(nxt, m_nxt, which ^ 1);
     } else {
-      if (!turn) M::fetch(Pl, A, nxt.visit, m_nxt, pn);
-      M::compute(Pl, A, cur.visit, cur.c0, cur.n, lane, m_cur, buf(which), pv, cache, cur.l & 1);
+      if (!turn) M::template fetch<false>(Pl, A, nxt.visit, m_nxt, pn);
+      M::template compute<false>(Pl, A, cur.visit, cur.c0, cur.n, lane, m_cur, buf(which), pv, cache, cur.l & 1);
       __syncwarp();
       if (turn) {  // this warp's factors and contributions, for bulk copies and other teams
         __threadfence();
@@ -1486,7 +1546,7 @@ __device__ void run_task(const DevPlan& Pl, const typename M::Args& A, const Tas
         __syncwarp();
         if (!done) stage(nxt, m_nxt, which ^ 1);
       } else if (!done) {
-        M::fetch(Pl, A, nxt.visit, m_nxt, pn);
+        M::template fetch<false>(Pl, A, nxt.visit, m_nxt, pn);
       }
       __syncthreads();
       if (done) return;
@@ -1524,12 +1584,12 @@ __device__ void run_task_alone(const DevPlan& Pl, const typename M::Args& A, con
     m_cur = m_nxt;
     pv = pn;
     M::stage(Pl, A, cur.visit, m_cur, cur.n, lane, smem);
-    M::fetch(Pl, A, cur.visit, m_cur, pv);
+    M::template fetch<true>(Pl, A, cur.visit, m_cur, pv);
     nxt = tab.next(cur, ve, lane);
     const RawMeta<M::kPacked, P> r_nxt = meta(nxt);
     cp_wait_all();
     __syncwarp();
-    M::compute(Pl, A, cur.visit, cur.c0, cur.n, lane, m_cur, smem, pv, cache, cur.l & 1);
+    M::template compute<true>(Pl, A, cur.visit, cur.c0, cur.n, lane, m_cur, smem, pv, cache, cur.l & 1);
     __syncwarp();
     M::copy_out(Pl, A, cur.visit, m_cur, cur.n, lane, smem);
     __syncwarp();
