@@ -741,7 +741,7 @@ struct FactorMode {
   __device__ static double2* factor_block(const DevPlan& Pl) { return static_cast<double2*>(Pl.ff4); }
   // the reciprocal pivots of the last full elimination: the workspace the other placement's factor would use
   __device__ static T* reciprocals(const DevPlan& Pl) { return static_cast<T*>(kBF ? Pl.fac : Pl.ff4); }
-  static constexpr bool kKeepRcp = kYG && kCable && !kReuse;
+  __device__ static bool keeps_rcp(const Args&) { return kYG && kCable && !kReuse; }
 
   // Section 1's implicit-Euler system, each part in the fewest operations: the
   // diagonal less all its edges, s (1 + theta dt g), and the right-hand side
@@ -936,6 +936,7 @@ struct FactorMode {
 #pragma unroll
     for (int h = 0; h < P; ++h) first_row[h] = m.p[h].len > 0 ? L - m.p[h].len : kL;
     if (visit == 0) {
+      const bool keep_rcp = keeps_rcp(A);
       T* rcp_block = kBF ? reciprocals(Pl) + m.blk : nullptr;
       // per piece: the eliminated pivot (cable: E) and right-hand side of the
       // current row, its coupling (re-using a factor: its g) and stored
@@ -995,10 +996,10 @@ struct FactorMode {
               bf[q].y = y;
             else
               bf[q] = make_double2(f, y);
-            if (kKeepRcp) rcp_block[q] = rr;
+            if (keep_rcp) rcp_block[q] = rr;
           } else {
             if (!kReuse) sd[i] = f;
-            if (kKeepRcp) su[i] = rr;
+            if (keep_rcp) su[i] = rr;
             sb[i] = y;
           }
         } else {
@@ -1152,7 +1153,7 @@ struct FactorMode {
     }
     T* fac = static_cast<T*>(Pl.fac);
     T* rc = reciprocals(Pl);
-    const bool keep_fac = visit == 0 && !kReuse, keep_rcp = visit == 0 && kKeepRcp;
+    const bool keep_fac = visit == 0 && !kReuse, keep_rcp = visit == 0 && keeps_rcp(A);
     if (kPk) {
       const int e = tab[kL];
 #pragma unroll 1
