@@ -193,6 +193,14 @@ hines_status hines_plan_export_tasks(hines_plan_t plan, int64_t *branch_task, in
                                      int64_t *task_order);
 
 /*
+ * How much longer a solve's first launch (whole cells, subtrees' eliminations,
+ * top parts) takes on `teams` runners than on `lone` ones, in chunks of work:
+ * the figure by which a call chooses between teams of two warps and lone
+ * warps.  Also on host-only plans.  No paper counterpart.
+ */
+hines_status hines_plan_team_stretch(hines_plan_t plan, int64_t teams, int64_t lone, double *stretch);
+
+/*
  * The solver layout (Section 5: the data of the branches a warp solves
  * together, interleaved so that each step reads one contiguous run).  Every
  * chunk of a warp task owns a block starting on a multiple of 4 slots.  With

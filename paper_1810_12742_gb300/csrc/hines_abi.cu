@@ -168,6 +168,10 @@ hines_status upload(hines_plan_t p) {
   D.n_unknowns = H.n_unknowns;
   D.n_branches = (int64_t)nb;
   if (hines::prepare_unit_kernels(D) != cudaSuccess) return HINES_ERR_CUDA;
+  auto set_stretch = [&](hines::RunnerGrid& g) { g.stretch = H.team_stretch(g.teams, 2 * (int64_t)g.ctas); };
+  for (auto& g : D.grid) set_stretch(g);
+  for (auto& g : D.grid_nf) set_stretch(g);
+  set_stretch(D.grid_refine);
   // A copy from pageable memory returns once its bytes are staged, maybe before
   // they are on the device, and streams that do not block on the legacy stream
   // are not ordered after it: the plan is handed out only when all of it is there.
@@ -323,6 +327,16 @@ hines_status hines_plan_export_tasks(hines_plan_t p, int64_t* branch_task, int64
   }
   if (task_order)
     for (size_t b = 0; b < H.torder.size(); ++b) task_order[b] = H.torder[b];
+  return HINES_OK;
+}
+
+hines_status hines_plan_team_stretch(hines_plan_t p, int64_t teams, int64_t lone, double* stretch) {
+  if (!p || teams < 1 || lone < 1 || !stretch) return HINES_ERR_INVALID_ARG;
+  try {
+    *stretch = p->host.team_stretch(teams, lone);
+  } catch (const std::bad_alloc&) {
+    return HINES_ERR_OOM;
+  }
   return HINES_OK;
 }
 

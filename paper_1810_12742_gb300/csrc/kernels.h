@@ -25,6 +25,14 @@ struct TaskRec {
   int32_t nlvl, id, code;
 };
 
+// Persistent grid sizes of a kernel kind: teams of two warps, CTAs of two warps
+// with a task each; and how much longer the batch's phase A is on that many
+// teams than on that many lone warps, both at one chunk a unit of time.
+struct RunnerGrid {
+  int teams = 1, ctas = 1;
+  double stretch = 1.0;
+};
+
 // Device copy of the host plan (pointers into one metadata allocation) and
 // the plan's workspace.
 struct DevPlan {
@@ -63,13 +71,12 @@ struct DevPlan {
   const longlong2* pk_meta = nullptr;     // [nb] per position: (chunk block offset, parent's solver-layout index)
   const int64_t* pk_perm = nullptr;       // [n_packed] natural index of each solver-layout slot, -1 for padding
   const int64_t* pk_edge = nullptr;       // [n_packed] natural index of each slot's coupling (pk_perm unless re-rooted)
-  // persistent grid sizes per kernel kind: teams of two warps (x), CTAs of two warps with a task each (y)
-  int2 grid[8] = {};
-  int2 grid_nf[4] = {};                        // the same for the FP64 kinds keeping the factor at natural positions
+  RunnerGrid grid[8];                          // per kernel kind
+  RunnerGrid grid_nf[4];                       // the FP64 kinds keeping the factor at natural positions
   int32_t fp64_blocks = 0;                     // 1: FP64 factors in block order (hines_plan_opts.fp64_factor)
   int32_t sms = 1;                             // multiprocessors of the plan's device
   int32_t per_lane = 2;                        // branch pieces per warp lane (the plan's lane mapping)
-  int2 grid_refine = {};                       // the same for the refinement steps
+  RunnerGrid grid_refine;                      // the refinement steps
   // workspace
   void* fac = nullptr;    // 8 bytes per natural or solver-layout slot: factor (FP64 / FP32 solves), FP32 working
                           // arrays (refine)

@@ -12,6 +12,7 @@
 #include "plan.h"
 
 #include <algorithm>
+#include <functional>
 #include <numeric>
 #include <queue>
 
@@ -600,6 +601,36 @@ int build_host_plan(int32_t n_cells, const int32_t* ncomp, const int32_t* parent
     }
   }
   return HINES_OK;
+}
+
+// Runners take phase A's entries in order, each the next when it is free; an
+// entry's time is its chunks (both visits of a whole cell's task) and two more
+// for starting it; whoever ends a cell's last subtree runs its top part too.
+// Far more entries than runners: the fluid limit.
+double HostPlan::team_stretch(int64_t teams, int64_t lone) const {
+  const int64_t ne = phase_off.empty() ? 0 : phase_off[1];
+  if (teams < 1 || lone <= teams || ne <= teams) return 1.0;
+  if (ne > 16 * teams) return (double)lone / (double)teams;
+  auto time = [&](int64_t runners) {
+    std::priority_queue<int64_t, std::vector<int64_t>, std::greater<int64_t>> free_at;
+    for (int64_t r = 0; r < std::min(runners, ne); ++r) free_at.push(0);
+    std::vector<int32_t> left = cell_nsub;
+    int64_t end = 0;
+    for (int64_t k = 0; k < ne; ++k) {
+      const int32_t t = phase_entry[(size_t)k] >> 2, code = phase_entry[(size_t)k] & 3;
+      int64_t at = free_at.top() + 2 + (int64_t)task_nlvl[(size_t)t] * (code == 0 ? 2 : 1);
+      free_at.pop();
+      if (code == 1) {
+        const size_t cell = (size_t)task_sub[2 * (size_t)t];
+        left[cell] -= task_sub[2 * (size_t)t + 1];
+        if (left[cell] == 0) at += 2 + 2 * (int64_t)task_nlvl[(size_t)cell_top_task[cell]];
+      }
+      free_at.push(at);
+      end = std::max(end, at);
+    }
+    return (double)end;
+  };
+  return time(teams) / time(lone);
 }
 
 }  // namespace hines

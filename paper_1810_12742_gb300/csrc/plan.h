@@ -71,6 +71,9 @@ struct HostPlan {
   // where the shorter piece has none).  So a warp reads a row as one
   // contiguous run, each lane its two values as one 8-byte word.  Blocks start
   // on multiples of kPackAlign compartments.
+  // Phase A's time on `teams` runners over its time on `lone`, in chunks.
+  double team_stretch(int64_t teams, int64_t lone) const;
+
   int64_t n_packed = 0;
   std::vector<int64_t> pk_blk;    // [nb] block offset of the chunk of each position
   std::vector<int64_t> pk_pcomp;  // [nb] solver-layout index of the parent branch's distal compartment, -1 at a root

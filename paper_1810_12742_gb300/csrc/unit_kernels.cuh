@@ -426,6 +426,9 @@ struct CompMode {
   // 414; phase A alone, 2370 entries 535 : 573; solver layout, whose copies are
   // bulk copies, 1197 381 : 412, 2629 665 : 601)
   static constexpr int kTeamShare = kPk ? 18 : 24;
+  // a team's speed at a chunk against a lone warp's (one task each: 1.15 to
+  // 1.26, solver layout 1.0 to 1.06)
+  static constexpr double kTeamSpeed = kPk ? 1.15 : 1.25;
   static_assert(kStageBytes % 16 == 0, "16-byte aligned buffers");
   using Bulk = BulkStage<kTab + 80>;
 
@@ -730,6 +733,10 @@ struct FactorMode {
   // phase A alone, 2715 235 : 329; re-using a factor: 2184 2511 : 2817, 2700
   // 5731 : 5727)
   static constexpr int kTeamShare = kReuse ? 40 : 32;
+  // one task each: FP64 and FP32 1.15 to 1.29, cable 1.18 to 1.23, re-using a
+  // factor 1.32; stretch 1.31 (1024 uneven cells): FP64 929 : 977, cable step
+  // 1514 : 1371
+  static constexpr double kTeamSpeed = kCable && !kReuse ? 1.25 : sizeof(T) == 4 ? 1.3 : 1.35;
   // the factor block is staged by bulk copies
   static constexpr bool kBulk = kBF;
   static_assert(kStageBytes % 16 == 0, "16-byte aligned buffers");
@@ -1212,9 +1219,10 @@ struct RefineMode {
   static constexpr int kTeamBytes = 2 * kStageBytes + kCacheBytes;
   static constexpr int kWarpBytes = kStageBytes + kCacheBytes;
   static constexpr int kMinBlocks = teams_per_sm(kTeamBytes, 10), kMinBlocksAlone = teams_per_sm(2 * kWarpBytes, 10);
-  // the same, always (us a solve of one step: 700 entries 625 : 958, 2700 1610
-  // : 2093): the copies outweigh the short arithmetic
+  // the same, by stretch only (one step with its FP32 solve: 1.0 139 : 179,
+  // 1.22 1108 : 1201, 1.32 901 : 947, 1.5 1324 : 1212, 1.9 3091 : 3103)
   static constexpr int kTeamShare = 1 << 20;
+  static constexpr double kTeamSpeed = 1.45;
   __device__ static void init_buffer(unsigned char*) {}
 
   // what the chunk needs of earlier chunks: the parent's x (visit 0), the
@@ -1698,9 +1706,9 @@ cudaError_t grid_of(const DevPlan& P, int* grid) {
 }
 // persistent grid sizes of both kernels of a mode: teams, and CTAs of two lone warps
 template <class M>
-cudaError_t grid_of(const DevPlan& P, int2* grid) {
-  cudaError_t e = grid_of<M, true>(P, &grid->x);
-  return e == cudaSuccess ? grid_of<M, false>(P, &grid->y) : e;
+cudaError_t grid_of(const DevPlan& P, RunnerGrid* grid) {
+  cudaError_t e = grid_of<M, true>(P, &grid->teams);
+  return e == cudaSuccess ? grid_of<M, false>(P, &grid->ctas) : e;
 }
 
 // The work counters and the cells' counts of finished subtrees are 0 when they
@@ -1715,7 +1723,7 @@ cudaError_t grid_of(const DevPlan& P, int2* grid) {
 // the last entry or finished the last subtree, a count that once went wrong
 // stayed wrong, and later calls left out entries or top parts silently.)
 template <class M>
-cudaError_t launch_phases(const DevPlan& P, const typename M::Args& A, int2 grid, cudaStream_t s) {
+cudaError_t launch_phases(const DevPlan& P, const typename M::Args& A, const RunnerGrid& grid, cudaStream_t s) {
   if (P.n_wtasks == 0) return cudaSuccess;
   const bool cut = P.phase_off[3] > P.phase_off[2];
   for (int phase = 0; phase < 3; ++phase) {
@@ -1724,16 +1732,24 @@ cudaError_t launch_phases(const DevPlan& P, const typename M::Args& A, int2 grid
     int runners;
     // Teams where one warp per entry leaves the chip idle anyway or a task's
     // own latency decides, lone warps, twice as many tasks at a time, where
-    // there are entries for them.  Phase A ends with the top parts, one after
-    // the other's chunks: the mode's share.  Phase C (subtrees'
-    // substitutions) has no such tail: teams while every entry has one (2306
-    // entries on 1824 teams 263 us, on lone warps 214).
-    const int share = phase == 0 ? M::kTeamShare : 16;
-    if ((int64_t)ne * 16 <= (int64_t)share * grid.x) {
-      runners = ne < grid.x ? ne : grid.x;
+    // there are entries for them.  Phase A ends with the longest chains of
+    // chunks, so more entries than teams may still do better on teams: up to
+    // the mode's share, and while phase A on the fewer teams is not longer, in
+    // chunks, than a team is faster at a chunk (RunnerGrid::stretch, the
+    // mode's kTeamSpeed).  Without the second bound 2000 equal tasks ran on 1216
+    // or 1824 teams in two rounds where lone warps take one: 2000 stars of 3000
+    // compartments FP64 3.22 ms, by lone warps 1.79, compensated 2.60 and 1.52;
+    // a million cells of 12 compartments 731 and 536, 501 and 399 us.  Phase C
+    // (subtrees' substitutions) has no such tail: teams while every entry has
+    // one (2306 entries on 1824 teams 263 us, on lone warps 214).
+    const bool teams = phase == 0 ? (int64_t)ne * 16 <= (int64_t)M::kTeamShare * grid.teams &&
+                                        grid.stretch <= M::kTeamSpeed
+                                  : ne <= grid.teams;
+    if (teams) {
+      runners = ne < grid.teams ? ne : grid.teams;
       k_units<M, true><<<runners, 64, cta_bytes<M, true>(), s>>>(P, A, phase);
     } else {
-      const int ctas = (ne + 1) / 2 < grid.y ? (ne + 1) / 2 : grid.y;
+      const int ctas = (ne + 1) / 2 < grid.ctas ? (ne + 1) / 2 : grid.ctas;
       runners = 2 * ctas;
       k_units<M, false><<<ctas, 64, cta_bytes<M, false>(), s>>>(P, A, phase);
     }
@@ -1781,7 +1797,7 @@ struct UnitKernels {
     if (e == cudaSuccess) e = grid_of<PkF32>(P, &P.grid[5]);
     if (e == cudaSuccess) e = grid_of<PkComp>(P, &P.grid[6]);
     if (e == cudaSuccess) e = grid_of<PkCable>(P, &P.grid[7]);
-    int2 g_reuse;  // same footprint as the plain modes
+    RunnerGrid g_reuse;  // same footprint as the plain modes
     if (e == cudaSuccess) e = grid_of<CableReuse>(P, &g_reuse);
     if (e == cudaSuccess) e = grid_of<PkCableReuse>(P, &g_reuse);
     if (e == cudaSuccess) e = grid_of<R32to2>(P, &P.grid_refine);

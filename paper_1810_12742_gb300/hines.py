@@ -30,7 +30,7 @@ HINES_F32 = 1
 
 EXPORTS = [
     "hines_plan_create", "hines_plan_destroy", "hines_plan_layout", "hines_plan_info", "hines_plan_export",
-    "hines_plan_export_tasks",
+    "hines_plan_export_tasks", "hines_plan_team_stretch",
     "hines_solve", "hines_solve_compensated", "hines_solve_refine", "hines_cable_step", "hines_cable_solve", "hines_grad_du",
     "hines_cable_adjoint_step", "hines_cable_loss_seed", "hines_cable_loss_accumulate", "hines_plan_status",
     "hines_status_string",
@@ -78,6 +78,7 @@ def lib():
             L.hines_plan_info.argtypes = [vp, ctypes.POINTER(PlanInfo)]
             L.hines_plan_export.argtypes = [vp, vp, vp, vp, vp, vp, vp]
             L.hines_plan_export_tasks.argtypes = [vp, vp, vp, vp]
+            L.hines_plan_team_stretch.argtypes = [vp, ctypes.c_int64, ctypes.c_int64, ctypes.POINTER(f64)]
             L.hines_solve.argtypes = [vp, i32, vp, vp, vp, vp]
             L.hines_solve_refine.argtypes = [vp, vp, vp, vp, vp, i32, vp, vp]
             L.hines_solve_compensated.argtypes = [vp, vp, vp, vp, vp, vp]
@@ -206,6 +207,14 @@ class Plan:
         _check(lib().hines_plan_export_tasks(self._h, _np_ptr(out["branch_task"]), _np_ptr(out["branch_kind"]),
                                              _np_ptr(out["task_order"])), "hines_plan_export_tasks")
         return out
+
+    def team_stretch(self, teams: int, lone: int) -> float:
+        """hines_plan_team_stretch: a solve's first launch on `teams` runners
+        over the same on `lone`, in chunks of work."""
+        out = ctypes.c_double()
+        _check(lib().hines_plan_team_stretch(self._h, int(teams), int(lone), ctypes.byref(out)),
+               "hines_plan_team_stretch")
+        return out.value
 
     def export_packed(self) -> np.ndarray:
         """Natural index held by each solver-layout slot (-1: padding)."""
