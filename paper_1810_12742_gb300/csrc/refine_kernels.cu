@@ -97,25 +97,55 @@ __device__ __forceinline__ double warp_max(double v) {
   return v;
 }
 
-// One block per cell: the cell's largest correction of this step from the
-// per-branch maxima; HINES_WARN_REFINE when it grew since the last step.  (A
-// warp per cell loaded a large cell's 9000 maxima in 280 turns: two refinement
-// steps on 301 cells 1.80 ms, with a block per cell 1.61 ms.)
-__global__ void __launch_bounds__(256) k_growth(DevPlan P, const float* __restrict__ bcorr, double* __restrict__ prev) {
-  __shared__ double part[8];
-  for (int64_t c = blockIdx.x; c < P.n_cells; c += gridDim.x) {
-    double m = 0.0;
-    for (int64_t br = P.cell_br_off[c] + threadIdx.x; br < P.cell_br_off[c + 1]; br += 256)
-      m = fmax(m, widen(bcorr[br]));
-    m = warp_max(m);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int k = 1; k < 8; ++k) m = fmax(m, part[k]);
-      if (m > prev[c]) atomicMax(P.status, (int)HINES_WARN_REFINE);
-      prev[c] = m;
+// The cell's largest correction of this step from the per-branch maxima;
+// HINES_WARN_REFINE when it grew since the last step.  A block takes `per`
+// (1..8) consecutive cells at a time, a warp for each of up to kGrowthWarp
+// branches, the whole block for a larger one.  (A warp per cell whatever its
+// size loaded a large cell's 9000 maxima in 280 turns: two refinement steps on
+// 301 cells 1.80 ms, with a block for each 1.61; a block per cell whatever its
+// size left its warps idle on small ones: a step on a million cells of one
+// piece 3.4 ms, with a warp for each 0.66.)
+constexpr int kGrowthWarp = 256;
+__global__ void __launch_bounds__(256) k_growth(DevPlan P, const float* __restrict__ bcorr, double* __restrict__ prev,
+                                                int per) {
+  __shared__ unsigned part[8];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  // (the maxima are not negative, so their bits are ordered as they are)
+  auto largest = [&](int64_t lo, int64_t hi, int i, int step) {
+    unsigned m = 0u;
+    for (int64_t br = lo + i; br < hi; br += step) m = max(m, __float_as_uint(bcorr[br]));
+    return __reduce_max_sync(kFull, m);
+  };
+  auto check = [&](int64_t c, unsigned m, double last) {
+    const double now = widen(__uint_as_float(m));
+    if (now > last) atomicMax(P.status, (int)HINES_WARN_REFINE);
+    prev[c] = now;
+  };
+  for (int64_t c0 = (int64_t)blockIdx.x * per; c0 < P.n_cells; c0 += (int64_t)gridDim.x * per) {
+    const int64_t c1 = c0 + per < P.n_cells ? c0 + per : P.n_cells;
+    bool large = false;
+    if (c0 + w < c1) {
+      const int64_t c = c0 + w, lo = P.cell_br_off[c], hi = P.cell_br_off[c + 1];
+      large = hi - lo > kGrowthWarp;
+      if (!large) {
+        const double last = prev[c];
+        const unsigned m = largest(lo, hi, lane, 32);
+        if (lane == 0) check(c, m, last);
+      }
     }
-    __syncthreads();
+    if (!__syncthreads_or(large)) continue;
+    for (int64_t c = c0; c < c1; ++c) {
+      const int64_t lo = P.cell_br_off[c], hi = P.cell_br_off[c + 1];
+      if (hi - lo <= kGrowthWarp) continue;
+      const unsigned m = largest(lo, hi, threadIdx.x, 256);
+      if (lane == 0) part[w] = m;
+      __syncthreads();
+      if (w == 0) {
+        const unsigned all = __reduce_max_sync(kFull, lane < 8 ? part[lane] : 0u);
+        if (lane == 0) check(c, all, prev[c]);
+      }
+      __syncthreads();
+    }
   }
 }
 
@@ -174,7 +204,9 @@ cudaError_t launch_unit_refine(const DevPlan& P, const float* d, const float* u,
     e = launch_unit_refine_step(P, d, u, b, pairs ? static_cast<const void*>(x) : static_cast<const void*>(x0), pairs,
                                 x, step == steps, bcorr, s);
     if (e != cudaSuccess) break;
-    k_growth<<<grid_for(P, nc, 1), 256, 0, s>>>(P, bcorr, prev);
+    // 8 blocks to a multiprocessor, and cells enough for each of them before a block takes several
+    const int blocks_g = P.sms * 8, per = nc <= blocks_g ? 1 : nc >= 8 * blocks_g ? 8 : (nc + blocks_g - 1) / blocks_g;
+    k_growth<<<nc < blocks_g ? nc : blocks_g, 256, 0, s>>>(P, bcorr, prev, per);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && relres) {
