@@ -1219,10 +1219,11 @@ struct RefineMode {
   static constexpr int kTeamBytes = 2 * kStageBytes + kCacheBytes;
   static constexpr int kWarpBytes = kStageBytes + kCacheBytes;
   static constexpr int kMinBlocks = teams_per_sm(kTeamBytes, 10), kMinBlocksAlone = teams_per_sm(2 * kWarpBytes, 10);
-  // the same, by stretch only (one step with its FP32 solve: 1.0 139 : 179,
-  // 1.22 1108 : 1201, 1.32 901 : 947, 1.5 1324 : 1212, 1.9 3091 : 3103)
+  // the same, by stretch only (one step: 1.0 82 : 107, 1.22 727 : 802, 1.31 1042
+  // : 1235, 1.5 2065 : 2447, 886 : 886 and 202 : 194, 1.9 2008 : 2019, 2.0 1727 :
+  // 1317)
   static constexpr int kTeamShare = 1 << 20;
-  static constexpr double kTeamSpeed = 1.45;
+  static constexpr double kTeamSpeed = 1.6;
   __device__ static void init_buffer(unsigned char*) {}
 
   // what the chunk needs of earlier chunks: the parent's x (visit 0), the
