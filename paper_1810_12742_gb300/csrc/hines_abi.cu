@@ -52,7 +52,7 @@ hines_status upload(hines_plan_t p) {
     m.pcomp = pb < 0 ? -1 : H.br_first[(size_t)pb] + H.br_len[(size_t)pb] - 1;
     m.ppos = pb < 0 ? -1 : H.tpos[(size_t)pb];
     const int32_t cb = H.tchild_ptr[k], ce = H.tchild_ptr[k + 1];
-    m.nchild = (uint16_t)(ce - cb);
+    if (ce - cb >= 1 << 30) return HINES_ERR_INVALID_ARG;  // (30 bits hold the count)
     int32_t lo = INT32_MAX, hi = -1;
     bool xtask = false;
     for (int32_t q = cb; q < ce; ++q) {
@@ -63,7 +63,7 @@ hines_status upload(hines_plan_t p) {
     const bool contig = ce > cb && hi - lo + 1 == ce - cb;
     m.child0 = contig ? lo : ce > cb ? H.tchild[(size_t)cb] : 0;
     m.child1 = ce - cb == 2 ? (contig ? lo + 1 : H.tchild[(size_t)cb + 1]) : cb;
-    m.flags = (uint16_t)((contig ? 1 : 0) | (xtask ? 2 : 0));
+    m.nchild_flags = (uint32_t)(ce - cb) << 2 | (contig ? 1u : 0u) | (xtask ? 2u : 0u);
   }
   // solver layout: per position (block offset, parent's solver-layout index)
   std::vector<int64_t> pkm(2 * H.torder.size());

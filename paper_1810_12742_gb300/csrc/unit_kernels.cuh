@@ -118,7 +118,7 @@ struct Meta {
 };
 
 // The same as it lies in memory.  A chunk's records are loaded two chunks
-// ahead and unpacked only when they are first needed: taking the 16-bit fields
+// ahead and unpacked only when they are first needed: taking the packed fields
 // apart right after the load waited for it in every chunk (about 600 clocks
 // with one warp on the multiprocessor, 2000 to 2500 with all of them resident).
 // With the chunk table in registers, the first entries without an atomic and
@@ -169,9 +169,9 @@ __device__ __forceinline__ Meta<P> unpack_meta(const RawMeta<kPk, P>& r) {
     q.child0 = (int)b.y;
     q.child1 = (int)b.z;
     q.len = (int)(a.y >> 24);
-    q.nchild = (int)(b.w & 0xFFFFu);
-    q.ccontig = (int)((b.w >> 16) & 1u);
-    q.xtask = (int)(b.w >> 17);
+    q.nchild = (int)(b.w >> 2);
+    q.ccontig = (int)(b.w & 1u);
+    q.xtask = (int)((b.w >> 1) & 1u);
     m.xpre[h].d = 0.0;
     m.cpre[h][0] = m.cpre[h][1] = make_double2(0.0, 0.0);
   }
