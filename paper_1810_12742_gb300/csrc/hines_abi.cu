@@ -63,7 +63,7 @@ hines_status upload(hines_plan_t p) {
     const bool contig = ce > cb && hi - lo + 1 == ce - cb;
     m.child0 = contig ? lo : ce > cb ? H.tchild[(size_t)cb] : 0;
     m.child1 = ce - cb == 2 ? (contig ? lo + 1 : H.tchild[(size_t)cb + 1]) : cb;
-    m.nchild_flags = (uint32_t)(ce - cb) << 2 | (contig ? 1u : 0u) | (xtask ? 2u : 0u);
+    m.nchild_flags = (uint32_t)(ce - cb) | (contig ? 1u << 30 : 0u) | (xtask ? 1u << 31 : 0u);
   }
   // solver layout: per position (block offset, parent's solver-layout index)
   std::vector<int64_t> pkm(2 * H.torder.size());

@@ -13,8 +13,8 @@ struct __align__(16) BrMetaT {
   int32_t ppos;           // position of the parent branch, -1 for a cell's root branch
   int32_t child0;         // position of the first child
   int32_t child1;         // two children: position of the second; more: index of the first child in tchild
-  uint32_t nchild_flags;  // children, times 4; 1: they are positions child0 .. child0 + nchild - 1; 2: some child
-                          // is in another task (written by another warp in the same launch)
+  uint32_t nchild_flags;  // children (30 bits); bit 30: they are positions child0 .. child0 + nchild - 1; bit 31: some
+                          // child is in another task (written by another warp in the same launch)
 };
 
 // A task as the kernels run it: where its chunk boundaries start (tlvl_ptr),

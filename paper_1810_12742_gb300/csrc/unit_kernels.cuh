@@ -169,9 +169,9 @@ __device__ __forceinline__ Meta<P> unpack_meta(const RawMeta<kPk, P>& r) {
     q.child0 = (int)b.y;
     q.child1 = (int)b.z;
     q.len = (int)(a.y >> 24);
-    q.nchild = (int)(b.w >> 2);
-    q.ccontig = (int)(b.w & 1u);
-    q.xtask = (int)((b.w >> 1) & 1u);
+    q.nchild = (int)(b.w & 0x3FFFFFFFu);
+    q.ccontig = (int)((b.w >> 30) & 1u);
+    q.xtask = (int)(b.w >> 31);
     m.xpre[h].d = 0.0;
     m.cpre[h][0] = m.cpre[h][1] = make_double2(0.0, 0.0);
   }
