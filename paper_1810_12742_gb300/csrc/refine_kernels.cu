@@ -37,13 +37,10 @@ __global__ void k_widen(const float* __restrict__ xf, double* __restrict__ x, in
     x[i] = widen(xf[i]);
 }
 
-// Residual r = b - A x in FP64 for every compartment, two branches per warp
-// (branches are at most 16 long).  kStats = false: r rounded to FP32 into rf.
-// kStats = true: per branch max |r|, max row sum |A| and max |x| into bstat.
-template <bool kStats>
+// Residual r = b - A x in FP64, two branches per warp (branches are at most 16
+// long): per branch max |r|, max row sum |A| and max |x| into bstat.
 __global__ void k_residual(DevPlan P, const float* __restrict__ d, const float* __restrict__ u,
-                           const float* __restrict__ b, const double* __restrict__ x, float* __restrict__ rf,
-                           double* __restrict__ bstat) {
+                           const float* __restrict__ b, const double* __restrict__ x, double* __restrict__ bstat) {
   const int lane = threadIdx.x & 31, half = lane >> 4, t = lane & 15;
   const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -59,35 +56,32 @@ __global__ void k_residual(DevPlan P, const float* __restrict__ d, const float* 
       const int32_t pb = P.br_parent[br];
       const double xi = x[i], di = widen(d[i]);
       r = fma(-di, xi, widen(b[i]));
-      if (kStats) a = fabs(di);
+      a = fabs(di);
       const int64_t pi = t > 0 ? i - 1 : (pb >= 0 ? (int64_t)P.br_first[pb] + P.br_len[pb] - 1 : -1);
       if (pi >= 0) {
         const double ui = widen(u[i]);
         r = fma(-ui, x[pi], r);
-        if (kStats) a += fabs(ui);
+        a += fabs(ui);
       }
       if (t < len - 1) {
         const double un = widen(u[i + 1]);
         r = fma(-un, x[i + 1], r);
-        if (kStats) a += fabs(un);
+        a += fabs(un);
       } else {
         for (int32_t c = P.child_ptr[br]; c < P.child_ptr[br + 1]; ++c) {
           const int64_t fc = P.br_first[P.child[c]];
           const double uc = widen(u[fc]);
           r = fma(-uc, x[fc], r);
-          if (kStats) a += fabs(uc);
+          a += fabs(uc);
         }
       }
-      if (!kStats) rf[i] = (float)r;
       xa = fabs(xi);
     }
-    if (kStats) {
-      const double rm = half_max(fabs(r)), am = half_max(a), xm = half_max(xa);
-      if (vb && t == 0) {
-        bstat[3 * br] = rm;
-        bstat[3 * br + 1] = am;
-        bstat[3 * br + 2] = xm;
-      }
+    const double rm = half_max(fabs(r)), am = half_max(a), xm = half_max(xa);
+    if (vb && t == 0) {
+      bstat[3 * br] = rm;
+      bstat[3 * br + 1] = am;
+      bstat[3 * br + 2] = xm;
     }
   }
 }
@@ -210,7 +204,7 @@ cudaError_t launch_unit_refine(const DevPlan& P, const float* d, const float* u,
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && relres) {
-    k_residual<true><<<blocks_b, 256, 0, s>>>(P, d, u, b, x, nullptr, bstat);
+    k_residual<<<blocks_b, 256, 0, s>>>(P, d, u, b, x, bstat);
     k_relres<<<blocks_c, 256, 0, s>>>(P, bstat, relres);
     e = cudaGetLastError();
   }

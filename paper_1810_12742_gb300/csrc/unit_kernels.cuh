@@ -413,9 +413,6 @@ struct CompMode {
   static constexpr int kArr = 3 * G::kSlots * 4, kFac = G::kSlots * 16;
   static constexpr int kTab = kArr > kFac ? kArr : kFac;
   static constexpr int kStageBytes = kTab + 96;
-  // contiguous blocks (the factor block; d, u, b in the solver layout) are
-  // staged by bulk copies (BulkStage, its barrier after the row table)
-  static constexpr bool kBulk = true;
   // the caches of the two sweeps share their space
   static constexpr int kCslot = 0, kCx = 0, kCacheBytes = 2 * G::kChunk * 16;
   static constexpr int kTeamBytes = 2 * kStageBytes + kCacheBytes;
@@ -430,12 +427,12 @@ struct CompMode {
   // 1.26, solver layout 1.0 to 1.06)
   static constexpr double kTeamSpeed = kPk ? 1.15 : 1.25;
   static_assert(kStageBytes % 16 == 0, "16-byte aligned buffers");
+  // contiguous blocks (the factor block; d, u, b in the solver layout) are
+  // staged by bulk copies, the barrier after the row table
   using Bulk = BulkStage<kTab + 80>;
 
-  __device__ static bool bulk_staged(int visit) { return kBulk && (visit == 1 || kPk); }
-  __device__ static void init_buffer(unsigned char* buf) {
-    if (kBulk) Bulk::init(buf);
-  }
+  __device__ static bool bulk_staged(int visit) { return visit == 1 || kPk; }
+  __device__ static void init_buffer(unsigned char* buf) { Bulk::init(buf); }
   // what the chunk needs of earlier chunks that no cache holds
   template <bool kAlone>
   __device__ static void fetch(const DevPlan& Pl, const Args&, int visit, Meta<P>& m, const Prev& pv) {
@@ -455,12 +452,7 @@ struct CompMode {
     build_row_table<P>(m.L, lane, tab);
     const int e = tab[kL];
     if (visit == 1) {
-      if (kBulk) {
-        Bulk::template issue<1>(buf, lane, (unsigned)e * 16u, buf, static_cast<const float4*>(Pl.ff4) + m.blk);
-      } else {
-        stage_block(reinterpret_cast<float4*>(buf), static_cast<const float4*>(Pl.ff4), m.blk, e, lane);
-        cp_commit();
-      }
+      Bulk::template issue<1>(buf, lane, (unsigned)e * 16u, buf, static_cast<const float4*>(Pl.ff4) + m.blk);
       return;
     }
     float* sd = reinterpret_cast<float*>(buf);
@@ -468,24 +460,17 @@ struct CompMode {
     float* sb = su + G::kSlots;
     if (kPk) {
       const long long blk = __shfl_sync(kFull, m.p[0].first, 0);
-      if (kBulk) {
-        // whole 16-byte words: the block's padding (blocks start on multiples
-        // of 4 slots, and the layout's length is one) completes the last
-        Bulk::template issue<3>(buf, lane, (unsigned)((e + 3) & ~3) * 4u, sd, A.d + blk, su, A.u + blk, sb,
-                                A.b + blk);
-        return;
-      }
-      stage_block(sd, A.d, blk, e, lane);
-      stage_block(su, A.u, blk, e, lane);
-      stage_block(sb, A.b, blk, e, lane);
-    } else {
-      for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g) {
-        const int q = nidx<P>(row, i);
-        cp_async4(&sd[q], A.d + g);
-        cp_async4(&su[q], A.u + g);
-        cp_async4(&sb[q], A.b + g);
-      });
+      // whole 16-byte words: the block's padding (blocks start on multiples
+      // of 4 slots, and the layout's length is one) completes the last
+      Bulk::template issue<3>(buf, lane, (unsigned)((e + 3) & ~3) * 4u, sd, A.d + blk, su, A.u + blk, sb, A.b + blk);
+      return;
     }
+    for_chunk_elements(m, n, lane, [&](int i, int, int row, long long g) {
+      const int q = nidx<P>(row, i);
+      cp_async4(&sd[q], A.d + g);
+      cp_async4(&su[q], A.u + g);
+      cp_async4(&sb[q], A.b + g);
+    });
     cp_commit();
   }
 
