@@ -716,8 +716,8 @@ def main():
                 "h2d_bytes_per_step": 12 * n_job, "d2h_bytes_per_step": 8 * n_job, "max_rel_err": e2e_err,
                 "path": f"C-ABI hines_pipeline_solve_compensated (through hines.HostPipeline) on pinned host "
                         f"arrays: the batch cut into {args.e2e_pieces} runs of consecutive cells, each with its own "
-                        "plan; per run the host-to-device copies, the device solve and the device-to-host copy on "
-                        "three internal streams, overlapped"},
+                        "plan; the runs' host-to-device copies, device solves and device-to-host copies on up to "
+                        "eight internal streams, overlapped"},
         "clocks": clk.summary(),
         "gpu_launches": 2 * args.steps,
     }

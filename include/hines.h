@@ -98,10 +98,11 @@ typedef struct {
                               compartments; the other size class is the subtrees of larger cells):
                               0 as pack_compartments, a count, or -1 for Section 4's rule */
   int32_t fp64_factor;     /* where the FP64 solves and cable steps keep their factor between the
-                              elimination and the substitution: 1 at natural positions (the
-                              reciprocal pivot in the workspace, the eliminated right-hand side in
-                              place), 2 in the chunks' block order (both as one 16-byte pair,
-                              staged back by bulk copies: faster on large batches, slower on
+                              elimination and the substitution, per compartment the coupling and
+                              the right-hand side over the eliminated pivot: 1 at natural
+                              positions (the first in the workspace, the second in place), 2 in
+                              the chunks' block order (both as one 16-byte pair, staged back by
+                              bulk copies: faster on large batches, slower on
                               latency-bound small ones), 0 (default) 2 for batches of at least
                               50,331,648 compartments, else 1; other values HINES_ERR_INVALID_ARG.
                               Results are the same bit for bit */
@@ -478,8 +479,8 @@ hines_status hines_pipeline_info(hines_pipeline_t pipeline, int32_t *pieces, int
  *   d, u, b   host float[n_unknowns], not modified
  *   x_out     host double[n_unknowns], the solution
  * Per run: the three input copies on one internal stream, the device solve
- * on a second, the copy of x back on a third, joined by events; the work is
- * ordered after everything enqueued on `stream` before the call, and
+ * on one of up to six, the copy of x back on another, joined by events; the
+ * work is ordered after everything enqueued on `stream` before the call, and
  * `stream` waits for all of it (x_out is complete when the stream reaches
  * that point).  The transfers overlap only when the host arrays are
  * page-locked (cudaHostAlloc, cudaHostRegister, pinned torch tensors); with

@@ -89,9 +89,11 @@ static __device__ __noinline__ double rcp_fp64_pipe(double x) {
   const double e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
-// FP64 with FP32 and integer instructions only.  An FP64 instruction costs a
-// warp 75 scheduler clocks on this part (64 clocks of latency), an FP32 one 1
-// (4), so the three FP64 FMAs of the form above bound the eliminations.
+// FP64 with FP32 and integer instructions only.  An FP64 instruction takes 64
+// clocks on this part where one warp issues them (dependent or not), 76 a
+// scheduler where all four issue them back to back, an FP32 one 1 (4 of
+// latency), so the three FP64 FMAs of the form above (68 each: its seed leaves
+// gaps) bound the eliminations.
 // The mantissa m in [1, 2) is cut into xf (24 bits), x1 (24 bits) and x2 (5
 // bits); r is the hardware's FP32 reciprocal of xf, which lies in [0.5, 1] for
 // every xf and leaves a residual 1 - xf r below 2^-23 that one FMA gives
@@ -100,9 +102,9 @@ static __device__ __noinline__ double rcp_fp64_pipe(double x) {
 // r (e + e^2) is rounded to units of 2^-53, the last place of a result in
 // [0.5, 1), through two sums with large constants, and is added to r's bit
 // pattern as an integer.  Largest error seen over 25 million values: 0.50002
-// units of the last place.  Measured per warp: latency 243 -> 148 clocks,
-// throughput 204 -> 48 clocks; FP64 solve of 59M compartments with the copy
-// of b 2.13 -> 1.92 ms, cable step of 14M 1.56 -> 1.35 ms.
+// units of the last place.  Measured: one warp 210 -> 125 clocks, eight warps a
+// scheduler 204 -> 47 each; FP64 solve of 59M compartments with the copy of b
+// 2.13 -> 1.92 ms, cable step of 14M 1.56 -> 1.35 ms.
 // In two halves, so that a caller can place FP64 instructions that do not
 // depend on it between them.
 struct RcpHalf {

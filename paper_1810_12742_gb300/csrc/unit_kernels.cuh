@@ -2,8 +2,8 @@
 //
 // The planner cuts every cell into units -- whole small cells, or the top part
 // and the subtrees of a large cell -- and packs units into tasks.  A runner --
-// a team of two warps, or a lone warp in launches with many entries -- owns a
-// task and walks its chunks (Hu's list schedule of the task's pieces, at most
+// a team of two warps, or a lone warp where teams would take more rounds of
+// tasks (launch_phases) -- owns a task and walks its chunks (Hu's list schedule of the task's pieces, at most
 // 32 * P pieces each, longest first): deepest chunk first for the
 // elimination, root-side chunk first for the substitution (Section 3).  In a
 // team one warp computes; the other moves data, so that copying a chunk's
@@ -663,8 +663,8 @@ struct CompMode {
 // operations, and nothing cancels where the leak is small next to a.
 //
 // The FP64 pipe and the latency of a row bound this mode: an FP64 instruction
-// takes 75 scheduler clocks per warp (64 clocks of latency), so a row holds as
-// few of them as possible (elimination 4, cable 5, substitution 1), and the
+// takes a scheduler 64 to 76 clocks (64 of latency), so a row holds as few of
+// them as possible (elimination 4, cable 5, substitution 1), and the
 // next row's inputs are read before the current row's results are written
 // (the compiler may not move them over the stores).
 // ============================================================================
@@ -714,8 +714,8 @@ struct FactorMode {
   static constexpr int kWarpBytes = kStageBytes + kCacheBytes;
   static constexpr int kMinBlocks = teams_per_sm(kTeamBytes, 10), kMinBlocksAlone = teams_per_sm(2 * kWarpBytes, 10);
   // the same (us; FP64: 1440 entries 262 : 318, 1514 668 : 764, 2184 376 :
-  // 392, 2260 586 : 628, 2707 542 : 509, 2755 954 : 953; FP32: 1514 195 : 236,
-  // phase A alone, 2715 235 : 329; re-using a factor: 2184 2511 : 2817, 2700
+  // 392, 2260 586 : 628, 2707 542 : 509, 2755 954 : 953; FP32: 1514 162 : 205,
+  // 2370 592 : 639, 2618 380 : 399; re-using a factor: 2184 2511 : 2817, 2700
   // 5731 : 5727)
   static constexpr int kTeamShare = kReuse ? 40 : 32;
   // one task each: FP64 and FP32 1.15 to 1.29, cable 1.18 to 1.23, re-using a

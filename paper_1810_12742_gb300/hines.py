@@ -476,8 +476,8 @@ class HostPipeline:
     """hines_pipeline_*: the compensated solve from host arrays, with the
     transfers overlapped.  The library cuts the batch into ``pieces`` runs of
     consecutive cells of about equal size, each with its own plan and device
-    buffers, and per run overlaps the host-to-device copies, the solve and the
-    copy back on three internal streams.  ``solve_compensated`` takes CPU
+    buffers, and overlaps the runs' host-to-device copies, solves and copies
+    back on up to eight internal streams.  ``solve_compensated`` takes CPU
     tensors in the natural layout of the whole batch (pinned, for the
     overlap) and enqueues the work after the current stream, which then waits
     for all of it.  plan_options go to every run's plan."""
