@@ -363,12 +363,12 @@ hines_status hines_cable_solve_packed(hines_plan_t plan, const double *s, const 
  * bit.  The caller guarantees that s, g, u, dt and theta are those of the last
  * full step or cable solve on this plan, in the same layout, and that no other
  * call has used the plan's workspace since (a hines_solve is such a call: it
- * leaves no reciprocals).  It pays in the solver layout at every size and in
- * the natural layout where the factor is kept at natural positions
- * (hines_plan_opts.fp64_factor); in the natural layout with block-order
- * factors it is slower than a full step (228M compartments: 8.2 against 7.4
- * ms; solver layout 4.7 against 6.2), since it gathers the reciprocals and
- * couplings one by one.  No paper counterpart (the paper solves each step
+ * leaves no reciprocals).  It pays in the solver layout at every size (228M
+ * compartments of uneven cells 4.7 against 6.3 ms).  In the natural layout
+ * with block-order factors (hines_plan_opts.fp64_factor) it gathers the
+ * reciprocals and couplings one by one and may lose to a full step (the same
+ * batch 8.3 against 7.5 ms; 60M compartments of one tree shape 3.5 against
+ * 4.1).  No paper counterpart (the paper solves each step
  * afresh; factor reuse is the constant-matrix special case of the passive
  * cable).
  *   solver_layout  0: natural-layout arrays (n_unknowns); 1: solver layout
